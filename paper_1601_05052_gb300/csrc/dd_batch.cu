@@ -244,6 +244,7 @@ dd_status configure(dd_batch_s *bt, const std::vector<dd_variant> &pv) {
         a.B = p->B;
         a.copies = t.d_copies;
         a.n_copies = t.n_copies;
+        a.copies_ahead = t.copies_ahead ? 1 : 0;
         a.offs = t.d_offs;
         a.bdesc = t.d_bdesc;
         a.n_blocks = t.n_blocks;

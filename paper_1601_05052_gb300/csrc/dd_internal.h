@@ -81,6 +81,7 @@ struct FwdTables {
     size_t smem_bytes = 0;       // dynamic shared memory of one CTA
     int4 *d_copies = nullptr;    // [n_dtiles][n_chunks][n_copies]
     int n_copies = 0;
+    bool copies_ahead = false;   // slots hold a later chunk's copies (kinds 0, 1, 5)
     // launch order of the one-shot kernel: time tiles fastest (true) or DM
     // tiles fastest (false, the default); chosen by dd_tune
     bool time_major = false;

@@ -331,6 +331,13 @@ dd_status build_fwd_tables(dd_plan_s *p, const dd_variant &v, FwdTables *out) {
     if (v.kind == 3)  // 3 partial-sum slots, each with the chunk's trial offsets
         p_bytes = size_t(3) * (size_t(t.p_elems) * 4 + size_t(cch / kSbGroup) * t.Dt * 2);
     t.smem_bytes = 128 + size_t(v.stages) * (t.stage_data_bytes + t.stage_offs_bytes) + p_bytes;
+    // kinds 0, 1 and 5: a slot also holds a later chunk's staging copies, if
+    // they fit (else the staging warp reads them from global memory)
+    if (!sb && t.smem_bytes + size_t(v.stages) * t.n_copies * 16 <= p->smem_optin) {
+        t.copies_ahead = true;
+        t.stage_offs_bytes += t.n_copies * 16;
+        t.smem_bytes += size_t(v.stages) * t.n_copies * 16;
+    }
     if (t.smem_bytes > p->smem_optin)
         return fail(DD_ERR_ARG, "variant needs more shared memory than the device has");
 
