@@ -81,8 +81,11 @@ typedef struct dd_stream_s *dd_stream;
  *         one series value per group (lane-strided); plus one producer warp.
  * kind 3: kind 2 with 4 dedicated builder warps (warp-specialised).
  * kind 4: kind 2 in CTAs of up to 16 trial warps (one CTA per SM).
- * kind 5: kind 0 that reuses the loaded operands for a trial whose delay in
- *         the channel equals the previous trial's.
+ * kind 5: kind 0 that serves several trials from the loaded operands: with 8
+ *         or 4 samples per thread, a trial whose delay in the channel equals
+ *         the previous trial's; with 14, 18 or 22 (two runs of consecutive
+ *         samples), every trial of the thread whose delay lies within the
+ *         window it holds in registers.
  * kind 6: kind 4 with one partial-sum slot and a second barrier per chunk,
  *         so that FP32 input fits chunks of 32 channels.
  * Results do not depend on the variant beyond FP32 summation order (8-bit
@@ -93,7 +96,10 @@ typedef struct {
     int32_t samples_per_thread;  /* samples accumulated per thread          */
     int32_t warps_dm;            /* warps along the DM axis of a CTA        */
     int32_t warps_time;          /* warps along the time axis of a CTA      */
-    int32_t chans_per_stage;     /* channels per pipeline stage: 4, 8, 16, 32 */
+    int32_t chans_per_stage;     /* channels per pipeline stage: 4, 8, 16, 32;
+                                  * 1 and 2 too for kind 0 with 8 x 8 outputs
+                                  * per thread and kind 5 with 14, 18 or 22
+                                  * samples, which may have 16 trial warps   */
     int32_t stages;              /* shared-memory pipeline depth (2..4)     */
 } dd_variant;
 

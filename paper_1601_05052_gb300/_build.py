@@ -16,7 +16,10 @@ CSRC = os.path.join(PKG, "csrc")
 OUT_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(OUT_DIR, "libdd.so")
 SOURCES = ["dd_plan.cpp", "dd_fwd.cu", "dd_adj.cu", "dd_tune.cpp", "dd_batch.cu", "dd_noalloc.cu",
-           "dd_stream.cpp", "dd_launches.cpp"]
+           "dd_stream.cpp", "dd_launches.cpp", "dd_default.cpp"]
+# (source, object suffix, flags): dd_kernels.cu once per input type
+UNITS = ([("dd_kernels.cu", "_%d" % i, ["-DDD_INST=%d" % i]) for i in range(5)]
+         + [(s, "", []) for s in SOURCES])
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -53,9 +56,10 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
                      "-I", os.path.join(ROOT, "include"), "--expt-relaxed-constexpr"]
     common += list(extra_flags)
 
-    def compile_one(src):
-        obj = os.path.join(obj_dir, os.path.splitext(src)[0] + ".o")
-        cmd = [nvcc] + common + ["-x", "cu", "-c", os.path.join(CSRC, src), "-o", obj]
+    def compile_one(unit):
+        src, suffix, flags = unit
+        obj = os.path.join(obj_dir, os.path.splitext(src)[0] + suffix + ".o")
+        cmd = [nvcc] + common + flags + ["-x", "cu", "-c", os.path.join(CSRC, src), "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("nvcc failed for %s:\n%s\n%s" % (src, " ".join(cmd), r.stderr))
@@ -63,8 +67,8 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
             print(r.stderr)
         return obj
 
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        objs = list(ex.map(compile_one, SOURCES))
+    with cf.ThreadPoolExecutor(max_workers=len(UNITS)) as ex:
+        objs = list(ex.map(compile_one, UNITS))
     tmp = LIB + ".%d.tmp" % os.getpid()
     cmd = [nvcc] + ARCH + ["-shared", "-cudart", "shared", "-o", tmp] + objs
     r = subprocess.run(cmd, capture_output=True, text=True)

@@ -25,94 +25,18 @@
 
 #include "dd_fwd_tile.cuh"
 #include "dd_internal.h"
+#include "dd_kernels.h"
 
 namespace dd {
 
-constexpr int kMaxBatchPlans = 16;
-
-struct BatchArgs {
-    const FwdArgs *args;  // [n], device
-    int n, stages;
-    long long item_start[kMaxBatchPlans + 1];
-    unsigned long long *counter;
-};
-
-template <int KIND, typename T, int DPT, int SPT>
-__global__ void __launch_bounds__(fwd_max_threads(KIND), fwd_min_blocks(KIND, DPT, SPT))
-    dd_fwd_persistent_kernel(const BatchArgs ba) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    // The item number alternates between two words: thread 0 writes the
-    // next one while a warp that is still leaving the previous tile may not
-    // yet have read the current one (a tile with no more chunks than stages
-    // lets the staging warp run ahead of the others).
-    __shared__ long long s_item[2];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem);
-    const volatile int *gave_up = reinterpret_cast<const volatile int *>(&bars[7]);
-    fwd_init_barriers<KIND>(bars, ba.stages);
-    uint32_t kbase = 0;
-    const long long n_items = ba.item_start[ba.n];
-    for (int it = 0;; it ^= 1) {
-        // a CTA that gave up a wait takes no further items
-        if (threadIdx.x == 0)
-            s_item[it] = *gave_up ? n_items : (long long)atomicAdd(ba.counter, 1ull);
-        __syncthreads();
-        const long long item = s_item[it];
-        if (item >= n_items) break;
-        int i = 0;
-        while (item >= ba.item_start[i + 1]) ++i;
-        const FwdArgs a = ba.args[i];
-        long long loc = item - ba.item_start[i];
-        const int dtile = int(loc % a.n_dtiles);
-        loc /= a.n_dtiles;
-        const int ttile = int(loc % a.n_ttiles);
-        const int b = int(loc / a.n_ttiles);
-        fwd_tile_any<KIND, T, DPT, SPT>(a, dtile, ttile, b, bars, smem + 128, kbase);
-    }
-}
-
 namespace {
-
-struct PersistentFn {
-    const void *fn = nullptr;
-    int (*occupancy)(int block, size_t smem) = nullptr;
-};
-
-// Raises the kernel's dynamic shared-memory limit to smem if it is lower (never
-// lowers it: another batch's captured graph may launch the same kernel with
-// more) and returns its resident CTAs per SM at (block, smem).
-template <int KIND, typename T, int DPT, int SPT>
-int occupancy_t(int block, size_t smem) {
-    cudaFuncAttributes fa{};
-    if (cudaFuncGetAttributes(&fa, dd_fwd_persistent_kernel<KIND, T, DPT, SPT>) != cudaSuccess)
-        return 0;
-    if (size_t(fa.maxDynamicSharedSizeBytes) < smem &&
-        cudaFuncSetAttribute(dd_fwd_persistent_kernel<KIND, T, DPT, SPT>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
-        return 0;
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &n, dd_fwd_persistent_kernel<KIND, T, DPT, SPT>, block, smem) != cudaSuccess)
-        return 0;
-    return n;
-}
-
-template <typename T>
-PersistentFn pick_persistent_t(int kind, int dpt, int spt) {
-#define DD_PICK(K_, D_, S_)                                                           \
-    if (kind == K_ && dpt == D_ && spt == S_)                                         \
-        return PersistentFn{(const void *)&dd_fwd_persistent_kernel<K_, T, D_, S_>, \
-                            &occupancy_t<K_, T, D_, S_>};
-    DD_FWD_KEYS(DD_PICK)
-#undef DD_PICK
-    return PersistentFn{};
-}
 
 PersistentFn pick_persistent(dd_dtype t, int kind, int dpt, int spt) {
     switch (t) {
-        case DD_F32: return pick_persistent_t<float>(kind, dpt, spt);
-        case DD_F16: return pick_persistent_t<__half>(kind, dpt, spt);
-        case DD_BF16: return pick_persistent_t<__nv_bfloat16>(kind, dpt, spt);
-        case DD_U8: return pick_persistent_t<uint8_t>(kind, dpt, spt);
+        case DD_F32: return pick_persistent_f32(kind, dpt, spt);
+        case DD_F16: return pick_persistent_f16(kind, dpt, spt);
+        case DD_BF16: return pick_persistent_bf16(kind, dpt, spt);
+        case DD_U8: return pick_persistent_u8(kind, dpt, spt);
     }
     return PersistentFn{};
 }
@@ -248,6 +172,7 @@ dd_status configure(dd_batch_s *bt, const std::vector<dd_variant> &pv) {
         a.offs = t.d_offs;
         a.bdesc = t.d_bdesc;
         a.n_blocks = t.n_blocks;
+        a.codes = t.d_codes;
         a.ttile0 = 0;
         a.dtile0 = 0;
         a.grid_tt = t.n_ttiles;
@@ -298,6 +223,28 @@ dd_status configure(dd_batch_s *bt, const dd_variant &v) {
     return s;
 }
 
+bool same_variant(const dd_variant &a, const dd_variant &b) {
+    return launch_compatible(a, b) && a.warps_dm == b.warps_dm &&
+           a.chans_per_stage == b.chans_per_stage;
+}
+
+// The plans' candidate variants by their modelled time over all plans.
+std::vector<RankedVariant> common_variants(const std::vector<dd_plan> &plans) {
+    std::vector<RankedVariant> common;
+    for (dd_plan p : plans)
+        for (const RankedVariant &r : ranked_variants(p))
+            if (std::none_of(common.begin(), common.end(),
+                             [&](const RankedVariant &x) { return same_variant(x.v, r.v); }))
+                common.push_back(RankedVariant{r.v, false, 0.0});
+    for (dd_plan p : plans) {
+        const DelaySteps st = delay_steps(p);
+        for (RankedVariant &r : common) r.us += model_us(p, st, r.v);
+    }
+    std::stable_sort(common.begin(), common.end(),
+                     [](const RankedVariant &a, const RankedVariant &b) { return a.us < b.us; });
+    return common;
+}
+
 // Work-list position of the caller's plan index u, or -1.
 int worklist_pos(const dd_batch_s *bt, int u) {
     for (size_t i = 0; i < bt->user_index.size(); ++i)
@@ -344,8 +291,11 @@ dd_status dd_batch_create(dd_batch *out, int32_t n, const dd_plan *plans) {
         dd_batch_destroy(bt);
         return cuda_fail(e, "cudaMalloc(batch)");
     }
-    // first plan's current variant if every plan fits it, else the defaults
-    dd_status s = configure(bt, plans[0]->fwd.v);
+    // The common variant with the smallest modelled time over all plans, among
+    // those that fit every plan; else any compiled variant that does.
+    dd_status s = DD_ERR_ARG;
+    const std::vector<RankedVariant> common = common_variants(bt->plans);
+    for (size_t i = 0; i < common.size() && s != DD_OK; ++i) s = configure(bt, common[i].v);
     if (s != DD_OK) {
         const int nv = dd_variant_count();
         for (int i = 0; i < nv && s != DD_OK; ++i) {
@@ -511,7 +461,9 @@ dd_status dd_batch_tune(dd_batch bt, int32_t budget_ms, dd_tune_report *rep) {
     const auto wall0 = std::chrono::steady_clock::now();
     const dd_variant start = bt->v;
     dd_variant best = start;
-    dd_status s = sweep_variants(budget_ms, flop, time_ms, &best, rep);
+    std::vector<dd_variant> extra;
+    for (const RankedVariant &r : common_variants(bt->plans)) extra.push_back(r.v);
+    dd_status s = sweep_variants(budget_ms, flop, time_ms, &best, rep, {}, extra);
     // Per-setup tile shapes: with the common kernel and staging depth fixed,
     // each plan in turn tries every split of the trial warps along DM and
     // time and every chunk size, keeping what shortens the whole launch by

@@ -10,29 +10,13 @@
 // CTAs then sweep one DM tile's rows, and the next DM tile, whose windows
 // are shifted by a few DM steps, finds them still in L2.
 #include <algorithm>
-#include <atomic>
 #include <limits>
 
 #include "dd_fwd_tile.cuh"
 #include "dd_internal.h"
+#include "dd_kernels.h"
 
 namespace dd {
-
-// LIVE: the plan has a live-chunk table (the adjoint's transposed gather,
-// FP32 only); tiles sum only their live chunks.
-template <int KIND, typename T, int DPT, int SPT, bool LIVE>
-__global__ void __launch_bounds__(fwd_max_threads(KIND), fwd_min_blocks(KIND, DPT, SPT))
-    dd_fwd_kernel(const FwdArgs a) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem);
-    fwd_init_barriers<KIND>(bars, a.stages);
-    uint32_t kbase = 0;
-    const int x = int(blockIdx.x);
-    const int dt = a.time_major ? x / a.grid_tt : x % a.grid_dt;
-    const int tt = a.time_major ? x % a.grid_tt : x / a.grid_dt;
-    fwd_tile_any<KIND, T, DPT, SPT, LIVE>(a, a.dtile0 + dt, a.ttile0 + tt, blockIdx.y, bars,
-                                          smem + 128, kbase);
-}
 
 // One CTA waits on an mbarrier that nothing arrives at, bounded by budget_ns.
 __global__ void dd_wait_timeout_kernel(int *err, unsigned long long budget_ns) {
@@ -81,80 +65,24 @@ void *mapped_host_ptr(void *p) { return const_cast<void *>(mapped_host_ptr(stati
 
 namespace {
 
-using FwdLaunchFn = cudaError_t (*)(const FwdArgs &, dim3, dim3, size_t, cudaStream_t);
-
-constexpr int kMaxDevices = 64;
-
-template <int KIND, typename T, int DPT, int SPT, bool LIVE>
-cudaError_t launch_fwd_t(const FwdArgs &a, dim3 grid, dim3 block, size_t smem, cudaStream_t st) {
-    // Make sure the kernel's dynamic shared-memory limit (set per device)
-    // covers smem, checking once per size increase; the limit is only ever
-    // raised, since other launches of the same kernel may need more.
-    static std::atomic<size_t> smem_set[kMaxDevices];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const bool cached = dev >= 0 && dev < kMaxDevices;
-    if (smem > 48 * 1024 && (!cached || smem > smem_set[dev].load())) {
-        cudaFuncAttributes fa{};
-        e = cudaFuncGetAttributes(&fa, dd_fwd_kernel<KIND, T, DPT, SPT, LIVE>);
-        if (e != cudaSuccess) return e;
-        if (size_t(fa.maxDynamicSharedSizeBytes) < smem) {
-            e = cudaFuncSetAttribute(dd_fwd_kernel<KIND, T, DPT, SPT, LIVE>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-            if (e != cudaSuccess) return e;
-        }
-        if (cached) smem_set[dev].store(smem);
-    }
-    dd_fwd_kernel<KIND, T, DPT, SPT, LIVE><<<grid, block, smem, st>>>(a);
-    return cudaGetLastError();
-}
-
-template <typename T, bool LIVE>
-FwdLaunchFn pick(int kind, int dpt, int spt) {
-#define DD_PICK(K_, D_, S_) \
-    if (kind == K_ && dpt == D_ && spt == S_) return &launch_fwd_t<K_, T, D_, S_, LIVE>;
-    DD_FWD_KEYS(DD_PICK)
-#undef DD_PICK
-    return nullptr;
-}
-
-// Live-chunk kernels exist for FP32 only (the adjoint's transposed gather).
-FwdLaunchFn pick_fn(dd_dtype t, int kind, int dpt, int spt, bool live) {
-    if (live) return t == DD_F32 ? pick<float, true>(kind, dpt, spt) : nullptr;
+// The kernel of a variant for a plan's input type (live: with live-chunk
+// ranges, FP32 only), or null functions if it is not compiled.
+FwdKernel pick_fwd(dd_dtype t, int kind, int dpt, int spt, bool live) {
+    if (live) return t == DD_F32 ? pick_fwd_f32_live(kind, dpt, spt) : FwdKernel{};
     switch (t) {
-        case DD_F32: return pick<float, false>(kind, dpt, spt);
-        case DD_F16: return pick<__half, false>(kind, dpt, spt);
-        case DD_BF16: return pick<__nv_bfloat16, false>(kind, dpt, spt);
-        case DD_U8: return pick<uint8_t, false>(kind, dpt, spt);
+        case DD_F32: return pick_fwd_f32(kind, dpt, spt);
+        case DD_F16: return pick_fwd_f16(kind, dpt, spt);
+        case DD_BF16: return pick_fwd_bf16(kind, dpt, spt);
+        case DD_U8: return pick_fwd_u8(kind, dpt, spt);
     }
-    return nullptr;
-}
-
-template <typename T, bool LIVE>
-const void *pick_kernel(int kind, int dpt, int spt) {
-#define DD_PICK_K(K_, D_, S_) \
-    if (kind == K_ && dpt == D_ && spt == S_) return (const void *)&dd_fwd_kernel<K_, T, D_, S_, LIVE>;
-    DD_FWD_KEYS(DD_PICK_K)
-#undef DD_PICK_K
-    return nullptr;
+    return FwdKernel{};
 }
 
 }  // namespace
 
 int fwd_resident_per_sm(const dd_plan_s *p, const FwdTables &t) {
     const int kind = t.v.kind, dpt = t.v.dm_per_thread, spt = t.v.samples_per_thread;
-    const void *k = nullptr;
-    if (t.d_live)
-        k = p->dtype == DD_F32 ? pick_kernel<float, true>(kind, dpt, spt) : nullptr;
-    else if (p->dtype == DD_F32)
-        k = pick_kernel<float, false>(kind, dpt, spt);
-    else if (p->dtype == DD_F16)
-        k = pick_kernel<__half, false>(kind, dpt, spt);
-    else if (p->dtype == DD_BF16)
-        k = pick_kernel<__nv_bfloat16, false>(kind, dpt, spt);
-    else
-        k = pick_kernel<uint8_t, false>(kind, dpt, spt);
+    const void *k = pick_fwd(p->dtype, kind, dpt, spt, t.d_live != nullptr).fn;
     if (!k) return 0;
     const int block = 32 * (t.v.warps_dm * t.v.warps_time + extra_warps(kind));
     // the query needs the kernel's dynamic shared-memory limit at least this
@@ -188,7 +116,7 @@ const std::vector<FwdKernelKey> &fwd_compiled_keys() {
 }
 
 bool fwd_variant_compiled(int kind, int dpt, int spt) {
-    return pick_fn(DD_F32, kind, dpt, spt, false) != nullptr;
+    return pick_fwd(DD_F32, kind, dpt, spt, false).fn != nullptr;
 }
 
 dd_status launch_forward(dd_plan_s *p, const FwdTables &t, const void *in, const void *w,
@@ -200,8 +128,9 @@ dd_status launch_forward(dd_plan_s *p, const FwdTables &t, const void *in, const
     if (n_dtiles < 0) n_dtiles = t.n_dtiles - dtile0;
     if (dtile0 < 0 || n_dtiles <= 0 || dtile0 + n_dtiles > t.n_dtiles)
         return fail(DD_ERR_ARG, "DM-tile range");
-    FwdLaunchFn fn = pick_fn(p->dtype, t.v.kind, t.v.dm_per_thread, t.v.samples_per_thread,
-                             t.d_live != nullptr);
+    FwdLaunchFn fn = pick_fwd(p->dtype, t.v.kind, t.v.dm_per_thread, t.v.samples_per_thread,
+                              t.d_live != nullptr)
+                         .launch;
     if (!fn) return fail(DD_ERR_UNSUPPORTED, "forward variant not compiled");
     FwdArgs a;
     a.in = in;
@@ -228,6 +157,7 @@ dd_status launch_forward(dd_plan_s *p, const FwdTables &t, const void *in, const
     a.offs = t.d_offs;
     a.bdesc = t.d_bdesc;
     a.n_blocks = t.n_blocks;
+    a.codes = t.d_codes;
     a.p_elems = t.p_elems;
     a.live = t.d_live;
     a.err = p->d_err;

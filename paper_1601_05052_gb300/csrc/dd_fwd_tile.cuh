@@ -36,9 +36,10 @@
 //  kind 3, warp-specialised sub-band: kind 2's arithmetic with 4 extra
 //    builder warps; mbarriers on the staging slots and on 3 partial-sum
 //    slots replace every CTA-wide barrier.
-//  kind 5, lane-strided with shared delays: kind 0, but a trial whose delay
-//    in the channel equals the previous trial's reuses the operands already
-//    in registers.
+//  kind 5, shared operands: kind 0, but operands in registers serve several
+//    trials: those whose delay in the channel equals the previous trial's, or
+//    (2 * odd samples per thread, see Window) every trial of the thread whose
+//    delay lies within a window of consecutive samples.
 //  kind 6, one-slot wide sub-band: kind 4 with a single partial-sum slot
 //    (one more barrier per chunk) and up to 8 groups per chunk, so that
 //    FP32 input fits 32-channel chunks.
@@ -58,7 +59,8 @@
 #define DD_FWD_KEYS(X)                                                                    \
     X(0, 2, 4) X(0, 4, 2) X(0, 4, 4) X(0, 8, 2) X(0, 8, 4) X(0, 4, 8) X(1, 8, 9) X(2, 4, 4) \
         X(2, 4, 8) X(2, 8, 4) X(2, 8, 2) X(3, 8, 4) X(3, 4, 8) X(3, 8, 2) X(4, 8, 4) X(4, 4, 8) \
-            X(5, 4, 8) X(5, 8, 4) X(6, 4, 8) X(0, 4, 16)
+            X(5, 4, 8) X(5, 8, 4) X(6, 4, 8) X(0, 4, 16) X(5, 4, 14) X(5, 4, 18) X(5, 4, 22) \
+                X(0, 8, 8)
 
 namespace dd {
 
@@ -120,6 +122,7 @@ struct FwdArgs {
     const uint16_t *offs;
     const int4 *bdesc;  // sub-band kinds: build blocks [n_dtiles][n_chunks][n_blocks]
     int n_blocks;       // sub-band kinds
+    const uint32_t *codes;  // register windows: [n_dtiles][n_chunks][warps_dm][cch]
     int p_elems;        // sub-band kinds
     // [n_dtiles][n_ttiles] {first, end} range of the chunks whose staged
     // windows reach the input's nonzero columns, for plans that declare zero
@@ -195,13 +198,16 @@ struct Stager {
     long long t0;
     const int4 *copies_k;  // this DM tile's staging copies
     const void *tab_k;    // kind 0/1: trial offsets; sub-band kinds: group offsets
-    const int4 *bdesc_k;  // sub-band kinds: this DM tile's build blocks
+    const void *tab2_k;   // second table: sub-band build blocks or window codes
     uint32_t tab_bytes;   // per chunk, both tables
     uint32_t tab1_bytes;  // per chunk, first table
     unsigned char *stage0;
     int stage_bytes;
     bool subband;
     int kc0;  // chunk k of the tile's loop is chunk kc0 + k of the plan
+
+    // Bytes of a slot's weights.
+    __device__ __forceinline__ int weight_bytes() const { return (a.cch * 4 + 15) & ~15; }
 
     // This lane's first staging copy of chunk k (copy `lane`; zero if none).
     __device__ __forceinline__ int4 desc(int k, int lane) const {
@@ -235,7 +241,9 @@ struct Stager {
         uint32_t total = copy_bytes(dsc);
 #pragma unroll
         for (int m = 16; m >= 1; m >>= 1) total += __shfl_xor_sync(0xffffffffu, total, m);
-        const uint32_t w_bytes = uint32_t((nch * 4 + 15) & ~15);
+        // the chunk's weights, from a 16-byte boundary on
+        const int w0 = c0 & ~3;
+        const uint32_t w_bytes = uint32_t(((c0 - w0 + nch) * 4 + 15) & ~15);
         const uint32_t d_bytes = ahead ? uint32_t(a.n_copies) * 16u : 0u;
         if (lane == 0) mbar_arrive_expect_tx(full, total + tab_bytes + w_bytes + d_bytes);
         __syncwarp();
@@ -244,20 +252,24 @@ struct Stager {
         if (lane == 0) {
             unsigned char *tb = sb + a.stage_data_bytes;
             if (!subband) {
-                bulk_g2s(tb, static_cast<const uint16_t *>(tab_k) + (size_t)c0 * a.Dt, tab_bytes,
+                bulk_g2s(tb, static_cast<const uint16_t *>(tab_k) + (size_t)c0 * a.Dt, tab1_bytes,
                          full);
             } else {
                 const int g0i = c0 / kSbG;
                 bulk_g2s(tb, static_cast<const uint16_t *>(tab_k) + (size_t)g0i * a.Dt,
                          tab1_bytes, full);
-                bulk_g2s(tb + tab1_bytes, bdesc_k + (size_t)(kc0 + k) * a.n_blocks,
-                         tab_bytes - tab1_bytes, full);
             }
-            // the chunk's weights; a 16-byte granule never crosses a page, so
-            // rounding the last chunk up stays inside the weight buffer's page
-            bulk_g2s(tb + tab_bytes, static_cast<const uint32_t *>(a.w) + c0, w_bytes, full);
+            if (tab_bytes > tab1_bytes) {
+                const uint32_t b2 = tab_bytes - tab1_bytes;
+                bulk_g2s(tb + tab1_bytes,
+                         static_cast<const unsigned char *>(tab2_k) + (size_t)(kc0 + k) * b2, b2,
+                         full);
+            }
+            // a 16-byte granule never crosses a page, so rounding the last
+            // chunk up stays inside the weight buffer's page
+            bulk_g2s(tb + tab_bytes, static_cast<const uint32_t *>(a.w) + w0, w_bytes, full);
             if (d_bytes)
-                bulk_g2s(tb + tab_bytes + a.cch * 4,
+                bulk_g2s(tb + tab_bytes + weight_bytes(),
                          copies_k + (size_t)(kc0 + k + ahead) * a.n_copies, d_bytes, full);
         }
     }
@@ -274,10 +286,11 @@ __device__ __forceinline__ Stager<T> make_stager(const FwdArgs &a, int dtile, in
                 a.copies + (size_t)dtile * ((a.C + a.cch - 1) / a.cch) * a.n_copies,
                 subband ? static_cast<const void *>(a.offs + (size_t)dtile * g_pad * a.Dt)
                         : static_cast<const void *>(a.offs + (size_t)dtile * a.C_pad * a.Dt),
-                subband ? a.bdesc + (size_t)dtile * ((a.C + a.cch - 1) / a.cch) * a.n_blocks
-                        : nullptr,
+                subband ? static_cast<const void *>(
+                              a.bdesc + (size_t)dtile * ((a.C + a.cch - 1) / a.cch) * a.n_blocks)
+                        : static_cast<const void *>(a.codes + (size_t)dtile * a.C_pad * a.warps_dm),
                 subband ? uint32_t(gpc) * a.Dt * 2 + uint32_t(a.n_blocks) * 16
-                        : uint32_t(a.cch) * a.Dt * 2,
+                        : uint32_t(a.cch) * (a.Dt * 2 + (a.codes ? a.warps_dm * 4 : 0)),
                 subband ? uint32_t(gpc) * a.Dt * 2 : uint32_t(a.cch) * a.Dt * 2,
                 stage0,
                 a.stage_data_bytes + a.stage_offs_bytes,
@@ -301,6 +314,40 @@ __device__ __forceinline__ void store_lane_strided(const FwdArgs &a, const Acc (
         for (int j = 0; j < SPT; ++j)
             if (32 * j < tmax) orow[32 * j] = acc[i][j];
     }
+}
+
+// Stores a thread's accumulators of the register-window kernels: each warp
+// turns one trial at a time around in its own 32 * SPT words of shared memory
+// (the staging slots, which nothing reads any more once every warp has passed
+// the barrier), so that the lanes' stores to global memory are coalesced.
+template <typename Acc, int DPT, int SPT>
+__device__ __forceinline__ void store_window(const FwdArgs &a, const Acc (&acc)[DPT][SPT], int dtile,
+                                             int b, long long t0, int wd, int wt, int lane, int warp,
+                                             volatile int *gave_up, unsigned char *stage0) {
+    constexpr int M = SPT / 2;
+    __syncthreads();
+    if (!*gave_up) {
+        Acc *buf = reinterpret_cast<Acc *>(stage0) + warp * 32 * SPT;
+#pragma unroll
+        for (int i = 0; i < DPT; ++i) {
+            const int d = dtile * a.Dt + wd * DPT + i;
+            if (d >= a.D) break;
+#pragma unroll
+            for (int j = 0; j < M; ++j) {
+                buf[lane * M + j] = acc[i][2 * j];
+                buf[32 * M + lane * M + j] = acc[i][2 * j + 1];
+            }
+            __syncwarp();
+            Acc *orow = static_cast<Acc *>(a.out) + ((long long)b * a.D + d) * a.S + t0 +
+                        wt * 32 * SPT + lane;
+            const long long tmax = a.S - t0 - wt * 32 * SPT - lane;
+#pragma unroll
+            for (int j = 0; j < SPT; ++j)
+                if (32 * j < tmax) orow[32 * j] = buf[32 * j + lane];
+            __syncwarp();
+        }
+    }
+    fence_proxy_async_smem();  // before the next tile's copies into these slots
 }
 
 // ------------------------------------------------------------------ kinds 0 and 1
@@ -400,6 +447,88 @@ struct RegWindow {
     }
 };
 
+// Register windows (kind 5 with 2 * odd samples per thread). Lane l of a warp
+// owns two runs of M = SPT / 2 consecutive samples, [l M, l M + M) and the
+// same 32 M samples later, for the DPT = 4 trials of its warp. Per channel it
+// loads the union window of its trials, M + (delay span) words per run, once
+// into registers and serves all four trials from it; which register holds a
+// trial's sample depends on the delay steps between the trials, so every
+// combination of steps within a band {b, b + 1} (all that an evenly spaced
+// DM grid produces) is a case of its own with compile-time positions,
+// entered by one warp-uniform jump per channel. The two runs make the
+// operands of the packed pair arithmetic: samples j of both runs sit in one
+// register pair whatever the delay. M is odd, so the lanes' loads are
+// conflict-free at every offset. Channels whose steps fit no case read one
+// word per add, like kind 0. Bound by issue slots and the shared-memory pipe
+// about equally (122 instructions per channel for 88 adds a thread at M = 11,
+// the pipe 68 % busy); two CTAs of 8 warps hide a tile's start and end better
+// than one of 16 (survey scale: 2.39 against 2.50 ms). Measured, FP32: 96 beams
+// x 64 channels x 64 trials x 4096 samples 0.187 ms (kind 5, equal delays) ->
+// 0.115; 16 beams x 512 channels x 1024 trials x 8192 samples 3.84 (kind 6) ->
+// 3.60 ms; survey scale 2.39 against kind 6's 2.34 ms.
+template <typename T, int SPT>
+struct Window {
+    using Acc = typename Elem<T>::Acc;
+    using Wt = typename Elem<T>::W;
+    static constexpr int DPT = 4, M = SPT / 2, H = 32 * M;
+
+    static __device__ __forceinline__ void add(Acc &a0, Acc &a1, Wt w, Acc x0, Acc x1) {
+        if constexpr (std::is_same<Acc, float>::value) {
+            fma2(a0, a1, w, w, x0, x1);
+        } else {
+            a0 += w * x0;
+            a1 += w * x1;
+        }
+    }
+
+    // acc[i][2 j + r] += w * s[d_i + j + r H], d = (0, S1, S1 + S2, S1 + S2 + S3)
+    template <int S1, int S2, int S3>
+    static __device__ __forceinline__ void serve(Acc (&acc)[DPT][SPT], const T *s, Wt w) {
+        constexpr int d[DPT] = {0, S1, S1 + S2, S1 + S2 + S3};
+#pragma unroll
+        for (int k = 0; k < M + d[DPT - 1]; ++k) {
+            const Acc x0 = Elem<T>::val(s[k]), x1 = Elem<T>::val(s[k + H]);
+#pragma unroll
+            for (int i = 0; i < DPT; ++i) {
+                const int j = k - d[i];
+                if (j >= 0 && j < M) add(acc[i][2 * j], acc[i][2 * j + 1], w, x0, x1);
+            }
+        }
+    }
+
+    static __device__ __forceinline__ void channel(Acc (&acc)[DPT][SPT], const T *sl, uint32_t code,
+                                                   const uint16_t *offs, Wt w) {
+        const T *s = sl + (code & 0xffffu);
+        switch (code >> 16) {
+#define DD_WIN_CASE(B_, K_)                                                          \
+    case 7 * B_ + K_:                                                                \
+        serve<B_ + (K_ & 1), B_ + ((K_ >> 1) & 1), B_ + ((K_ >> 2) & 1)>(acc, s, w); \
+        break;
+#define DD_WIN_BAND(B_)                                                         \
+    DD_WIN_CASE(B_, 0) DD_WIN_CASE(B_, 1) DD_WIN_CASE(B_, 2) DD_WIN_CASE(B_, 3) \
+    DD_WIN_CASE(B_, 4) DD_WIN_CASE(B_, 5) DD_WIN_CASE(B_, 6)
+            DD_WIN_BAND(0) DD_WIN_BAND(1) DD_WIN_BAND(2) DD_WIN_BAND(3) DD_WIN_BAND(4)
+            DD_WIN_CASE(4, 7)
+#undef DD_WIN_BAND
+#undef DD_WIN_CASE
+            case kWinNone: {
+                int o[DPT];
+                load_offsets<DPT>(offs, o);
+#pragma unroll
+                for (int i = 0; i < DPT; ++i) {
+                    const T *t = sl + o[i];
+#pragma unroll
+                    for (int j = 0; j < M; ++j)
+                        add(acc[i][2 * j], acc[i][2 * j + 1], w, Elem<T>::val(t[j]),
+                            Elem<T>::val(t[j + H]));
+                }
+                break;
+            }
+            default: __builtin_unreachable();
+        }
+    }
+};
+
 // Barriers: every kind uses full[s] = bars[s] (producer arrival + bytes) and
 // empty[s] = bars[8 + s]: one arrival per warp for kinds 0/1, one per chunk
 // for kind 2 (after its compute barrier), one per builder warp for kind 3,
@@ -439,6 +568,14 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs &a, int dtile, int ttile,
         KIND == 1, RegWindow<T, DPT, SPT>, LaneStrided<T, DPT, SPT, KIND == 5>>::type;
     using Acc = typename Elem<T>::Acc;
     using Wt = typename Elem<T>::W;
+    constexpr bool WIN = is_window(KIND, SPT);
+    // With two slots, a refill at the end of a chunk leaves no copy in flight
+    // during the next one; the kernels with the largest tiles, whose slots
+    // leave no room for a third, refill before they sum a chunk (LOFAR, 8
+    // trials x 4096 samples, two channels per slot: 2.94 -> 2.07 ms). The
+    // others keep the one place: a second copy of the staging code slows them
+    // (register windows at the survey scale: 2.41 -> 2.58 ms).
+    constexpr bool EARLY = KIND == 0 && DPT * SPT == 64;
     uint64_t *full = bars, *empty = bars + 8;
     volatile int *gave_up = reinterpret_cast<volatile int *>(&bars[7]);
     const uint32_t S = uint32_t(a.stages);
@@ -477,8 +614,25 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs &a, int dtile, int ttile,
     for (int i = 0; i < DPT; ++i)
 #pragma unroll
         for (int j = 0; j < SPT; ++j) acc[i][j] = Acc(0);
-    const int lb = P::lane_base(wt, lane);
+    const int lb = WIN ? wt * 32 * SPT + lane * (SPT / 2) : P::lane_base(wt, lane);
 
+    // stages the chunk that goes into chunk k - 1's slot (sb: chunk k's slot)
+    auto refill = [&](int k, const unsigned char *sb) {
+        const int kn = k - 1 + int(S);
+        if (k < 1 || kn >= n_chunks || warp != turn) return;
+        int4 dsc = make_int4(0, 0, 0, 0);
+        if (!a.copies_ahead)
+            dsc = st.desc(kn, lane);
+        else if (lane < a.n_copies)
+            dsc = reinterpret_cast<const int4 *>(sb + a.stage_data_bytes + st.tab_bytes +
+                                                 st.weight_bytes())[lane];
+        const int prev = slot ? slot - 1 : int(S) - 1;
+        // chunk k - 1's release: the same phase as its full barrier's
+        const uint32_t par = slot ? parity : parity ^ 1u;
+        const bool ok = mbar_wait_bounded(&empty[prev], par, a.err, kWaitBudgetNs, gave_up);
+        if (__all_sync(0xffffffffu, ok))
+            st.issue(kn, prev, dsc, &full[prev], lane, ahead(kn));
+    };
     for (int k = 0; k < n_chunks; ++k) {
         // A failed wait (or one that finds the CTA's give-up flag set) ends
         // the tile: the slot may hold a stale chunk, so nothing more is
@@ -490,31 +644,36 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs &a, int dtile, int ttile,
         const T *sdata = reinterpret_cast<const T *>(sb);
         const uint16_t *soffs =
             reinterpret_cast<const uint16_t *>(sb + a.stage_data_bytes) + wd * DPT;
-        const Wt *sw = reinterpret_cast<const Wt *>(sb + a.stage_data_bytes + st.tab_bytes);
-        const int nch = min(a.cch, a.C - (kr.x + k) * a.cch);
-        for (int cc = 0; cc < nch; ++cc) {
-            int o[DPT];
-            load_offsets<DPT>(soffs + cc * a.Dt, o);
-            P::channel(acc, sdata, lb, o, sw[cc]);
+        const int c0 = (kr.x + k) * a.cch, nch = min(a.cch, a.C - c0);
+        const Wt *sw =
+            reinterpret_cast<const Wt *>(sb + a.stage_data_bytes + st.tab_bytes) + (c0 & 3);
+        if (EARLY && S == 2) refill(k, sb);
+        if constexpr (WIN) {
+            const uint32_t *codes =
+                reinterpret_cast<const uint32_t *>(sb + a.stage_data_bytes + st.tab1_bytes) +
+                wd * a.cch;
+            uint32_t code = codes[0];
+            Wt wc = sw[0];
+#pragma unroll 1
+            for (int cc = 0; cc < nch; ++cc) {
+                // read one channel ahead, never past the chunk's last channel
+                const int cn = min(cc + 1, nch - 1);
+                const uint32_t code_next = codes[cn];
+                const Wt w_next = sw[cn];
+                Window<T, SPT>::channel(acc, sdata + lb, code, soffs + cc * a.Dt, wc);
+                code = code_next;
+                wc = w_next;
+            }
+        } else {
+            for (int cc = 0; cc < nch; ++cc) {
+                int o[DPT];
+                load_offsets<DPT>(soffs + cc * a.Dt, o);
+                P::channel(acc, sdata, lb, o, sw[cc]);
+            }
         }
-        const int kn = k - 1 + int(S);  // the chunk to stage into chunk k - 1's slot
-        const bool mine = k >= 1 && kn < n_chunks && warp == turn;
-        int4 dsc = make_int4(0, 0, 0, 0);
-        if (mine && !a.copies_ahead)
-            dsc = st.desc(kn, lane);
-        else if (mine && lane < a.n_copies)
-            dsc = reinterpret_cast<const int4 *>(sb + a.stage_data_bytes + st.tab_bytes +
-                                                 a.cch * 4)[lane];
+        if (!(EARLY && S == 2)) refill(k, sb);
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[slot]);
-        if (mine) {
-            const int prev = slot ? slot - 1 : int(S) - 1;
-            // chunk k - 1's release: the same phase as its full barrier's
-            const uint32_t par = slot ? parity : parity ^ 1u;
-            const bool ok = mbar_wait_bounded(&empty[prev], par, a.err, kWaitBudgetNs, gave_up);
-            if (__all_sync(0xffffffffu, ok))
-                st.issue(kn, prev, dsc, &full[prev], lane, ahead(kn));
-        }
         if (k >= 1 && ++turn == n_warps) turn = 0;
         if (++slot == int(S)) {
             slot = 0;
@@ -522,6 +681,10 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs &a, int dtile, int ttile,
         }
     }
     kbase += uint32_t(n_chunks);
+    if constexpr (WIN) {
+        store_window<Acc, DPT, SPT>(a, acc, dtile, b, t0, wd, wt, lane, warp, gave_up, stage0);
+        return;
+    }
     if (*gave_up) return;
 
     Acc *out = static_cast<Acc *>(a.out);

@@ -92,6 +92,9 @@ struct FwdTables {
     // 4 x 32 consecutive elements of one partial series, see
     // build_fwd_tables); p_elems the partial-sum buffer length of one chunk.
     int4 *d_bdesc = nullptr;
+    // register windows only: per (DM tile, chunk, trial warp, channel) the
+    // first trial's offset | step code << 16 (kWinNone: read d_offs)
+    uint32_t *d_codes = nullptr;
     int n_blocks = 0;
     int p_elems = 0;
     // largest delay of each DM tile (over its trials and all channels)
@@ -203,6 +206,21 @@ void free_adj_state(AdjState *a);
 dd_status launch_adjoint(dd_plan_s *p, const float *g, const float *w, const float *in,
                          float *gin, float *gw, cudaStream_t st);
 
+// Default variants (dd_default.cpp). Delay steps: how far a channel's delay
+// moves per trial, mean and largest over the channels.
+struct DelaySteps {
+    double mean = 0, max = 0;
+};
+DelaySteps delay_steps(const dd_plan_s *p);
+double model_us(const dd_plan_s *p, const DelaySteps &st, const dd_variant &v);
+struct RankedVariant {
+    dd_variant v;
+    bool time_major;
+    double us;  // modelled
+};
+// The candidate variants, fastest by the model first (they may not fit).
+std::vector<RankedVariant> ranked_variants(const dd_plan_s *p);
+
 bool aligned16(const void *p);
 
 // Tuning cache (DD_TUNE_CACHE): signature of a plan and a record of its
@@ -213,10 +231,13 @@ void cache_store(const std::string &key, const dd_variant &v, bool time_major);
 // Two-pass sweep of the variant grid (dd_tune.cpp). time_ms(v, &ms) sets ms
 // <= 0 for variants that do not fit; returns the fastest in *best.
 // between_passes (may be empty) sees pass 1's fastest variant before pass 2
-// starts (the plan tuner settles the launch order there).
+// starts (the plan tuner settles the launch order there). Pass 1 also times
+// the variants in `extra` (shapes outside the grid, such as the modelled
+// defaults).
 dd_status sweep_variants(int32_t budget_ms, double flop,
                          const std::function<dd_status(const dd_variant &, double *)> &time_ms,
                          dd_variant *best, dd_tune_report *rep,
-                         const std::function<dd_status(const dd_variant &)> &between_passes = {});
+                         const std::function<dd_status(const dd_variant &)> &between_passes = {},
+                         const std::vector<dd_variant> &extra = {});
 
 }  // namespace dd

@@ -5,7 +5,7 @@
 // kind 1: register windows; kind 2: sub-band partial series (groups of four
 // channels) with a producer warp; kind 3: kind 2 with warp-specialised
 // builders; kind 4: kind 2 in CTAs of up to 16 trial warps; kind 5: kind 0
-// with operand reuse between trials that share a channel's delay; kind 6:
+// with operand reuse between trials (equal delays, or register windows); kind 6:
 // kind 4 with one partial-sum slot and up to 8 groups per chunk, which lets
 // FP32 input stage 32 channels at a time.
 #pragma once
@@ -25,14 +25,30 @@ __host__ __device__ constexpr int extra_warps(int kind) {
 __host__ __device__ constexpr bool is_subband(int kind) {
     return kind == 2 || kind == 3 || kind == 4 || kind == 6;
 }
+// Register-window form of kind 5 (see dd_fwd_tile.cuh): 2 * odd samples per
+// thread in two runs of consecutive samples.
+__host__ __device__ constexpr bool is_window(int kind, int spt) {
+    return kind == 5 && spt % 4 == 2;
+}
+// Kernels whose CTAs may have 16 trial warps and stage 1 or 2 channels at a time:
+// the register windows and the lane-strided 8 x 8 form.
+__host__ __device__ constexpr bool is_wide(int kind, int dpt, int spt) {
+    return is_window(kind, spt) || (kind == 0 && dpt == 8 && spt == 8);
+}
+// Codes of the delay steps a register window serves: steps (s1, s2, s3)
+// between a thread's four trials with every step in {b, b + 1} are code 7 b +
+// (s1 - b) + 2 (s2 - b) + 4 (s3 - b), b < kWinBands (so all steps equal to b +
+// 1 are code 7 (b + 1)). Other steps: kWinNone.
+constexpr int kWinBands = 5;
+constexpr int kWinNone = 7 * kWinBands + 1;
 // Largest trial-warp count of a CTA.
-__host__ __device__ constexpr int max_trial_warps(int kind) {
-    return (kind == 4 || kind == 6) ? 16 : 8;
+__host__ __device__ constexpr int max_trial_warps(int kind, int dpt, int spt) {
+    return (kind == 4 || kind == 6 || is_wide(kind, dpt, spt)) ? 16 : 8;
 }
 // Launch bounds of the forward kernels: threads per CTA and resident CTAs
 // per SM that the register allocation must allow.
-__host__ __device__ constexpr int fwd_max_threads(int kind) {
-    return 32 * (max_trial_warps(kind) + extra_warps(kind));
+__host__ __device__ constexpr int fwd_max_threads(int kind, int dpt, int spt) {
+    return 32 * (max_trial_warps(kind, dpt, spt) + extra_warps(kind));
 }
 __host__ __device__ constexpr int fwd_min_blocks(int kind, int dpt, int spt) {
     return kind == 2 ? (dpt * spt <= 16 ? 3 : 2) : (kind == 3 ? 2 : 1);

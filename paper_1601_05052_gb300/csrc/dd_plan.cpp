@@ -54,11 +54,14 @@ dd_status replace_fwd_tables(dd_plan_s *p, FwdTables *cur, const FwdTables &next
 dd_status check_variant_shape(const dd_variant &v) {
     if (!fwd_variant_compiled(v.kind, v.dm_per_thread, v.samples_per_thread))
         return fail(DD_ERR_ARG, "variant (kind, dm_per_thread, samples_per_thread) not compiled");
-    if (v.warps_dm < 1 || v.warps_time < 1 || v.warps_dm * v.warps_time > max_trial_warps(v.kind))
+    if (v.warps_dm < 1 || v.warps_time < 1 ||
+        v.warps_dm * v.warps_time >
+            max_trial_warps(v.kind, v.dm_per_thread, v.samples_per_thread))
         return fail(DD_ERR_ARG,
-                    "variant warps_dm * warps_time must be in [1, 8] (kinds 4 and 6: [1, 16])");
-    if (v.chans_per_stage != 4 && v.chans_per_stage != 8 && v.chans_per_stage != 16 &&
-        v.chans_per_stage != 32)
+                    "variant warps_dm * warps_time must be in [1, 8] (wide kernels: [1, 16])");
+    const bool wide = is_wide(v.kind, v.dm_per_thread, v.samples_per_thread);
+    const int cch = v.chans_per_stage;
+    if (cch != 4 && cch != 8 && cch != 16 && cch != 32 && !(wide && (cch == 1 || cch == 2)))
         return fail(DD_ERR_ARG, "variant chans_per_stage must be 4, 8, 16 or 32");
     if (v.stages < 2 || v.stages > 4) return fail(DD_ERR_ARG, "variant stages must be 2..4");
     return DD_OK;
@@ -139,6 +142,29 @@ dd_status sb_chunk(const dd_plan_s *p, int d0, int d1, int Dt, int Ts, int c0, i
 
 }  // namespace
 
+// The word a register-window warp reads for one channel: its first trial's
+// offset and the code of the steps to the next trials' offsets (dd_kinds.h).
+// n: trials of the warp that exist; the others' sums are never stored, so
+// their steps are taken as the case needs them.
+uint32_t window_code(const uint16_t *o, int n) {
+    if (n <= 0) return 0;
+    int step[3] = {0, 0, 0}, lo = kWinBands + 1, hi = -1;
+    for (int i = 1; i < n; ++i) {
+        const int s = int(o[i]) - int(o[i - 1]);
+        if (s < 0 || s > kWinBands) return o[0] | uint32_t(kWinNone) << 16;
+        step[i - 1] = s;
+        lo = std::min(lo, s);
+        hi = std::max(hi, s);
+    }
+    if (n == 1) lo = hi = 0;
+    if (hi - lo > 1) return o[0] | uint32_t(kWinNone) << 16;
+    const int b = std::min(lo, kWinBands - 1);
+    int code = 7 * b;
+    for (int i = 0; i < 3; ++i)
+        if (i + 1 < n && step[i] > b) code += 1 << i;
+    return o[0] | uint32_t(code) << 16;
+}
+
 dd_status build_fwd_tables(dd_plan_s *p, const dd_variant &v, FwdTables *out) {
     dd_status s = check_variant_shape(v);
     if (s != DD_OK) return s;
@@ -155,6 +181,9 @@ dd_status build_fwd_tables(dd_plan_s *p, const dd_variant &v, FwdTables *out) {
     const bool sb = is_subband(v.kind);
     if (int64_t(t.n_ttiles) * t.n_dtiles > 0x7fffffffLL)
         return fail(DD_ERR_ARG, "too many tiles for this variant");
+    if (cch * t.Dt % 8 != 0 ||
+        (is_window(v.kind, v.samples_per_thread) && cch * v.warps_dm % 4 != 0))
+        return fail(DD_ERR_ARG, "too few trials for so few channels per stage");
     if (sb && t.Dt % 8 != 0) return fail(DD_ERR_ARG, "sub-band variants need 8 | DM tile");
     if (sb && v.kind != 6 && cch > 16 && p->dtype == DD_F32)
         return fail(DD_ERR_ARG, "sub-band kinds 2-4 with FP32 input stage at most 16 channels");
@@ -298,6 +327,20 @@ dd_status build_fwd_tables(dd_plan_s *p, const dd_variant &v, FwdTables *out) {
     std::vector<int4> copy_tab(copies.size() * size_t(t.n_copies), make_int4(0, 0, 0, 0));
     for (size_t i = 0; i < copies.size(); ++i)
         std::copy(copies[i].begin(), copies[i].end(), copy_tab.begin() + i * size_t(t.n_copies));
+    const bool win = is_window(v.kind, v.samples_per_thread);
+    std::vector<uint32_t> codes;
+    if (win) {
+        codes.assign(size_t(t.n_dtiles) * t.C_pad * v.warps_dm, 0);
+        for (int k = 0; k < t.n_dtiles; ++k)
+            for (int c = 0; c < p->C; ++c)
+                for (int wd = 0; wd < v.warps_dm; ++wd) {
+                    const int d0 = k * t.Dt + wd * v.dm_per_thread;
+                    const uint16_t *o = &offs[(size_t(k) * t.C_pad + c) * t.Dt +
+                                              wd * v.dm_per_thread];
+                    codes[((size_t(k) * n_chunks + c / cch) * v.warps_dm + wd) * cch + c % cch] =
+                        window_code(o, std::min(v.dm_per_thread, p->D - d0));
+                }
+    }
     std::vector<int4> bdesc;
     if (sb) {
         // Worker w of `parts` builds blocks w, w + parts, ... of a chunk in
@@ -321,7 +364,9 @@ dd_status build_fwd_tables(dd_plan_s *p, const dd_variant &v, FwdTables *out) {
                              t.n_blocks * 16 + cch * 4;
         t.p_elems = static_cast<int>(round_up(p_max + 64, 4));
     } else {
-        t.stage_offs_bytes = static_cast<int>(round_up(int64_t(cch) * t.Dt * 2, 16)) + cch * 4;
+        t.stage_offs_bytes = static_cast<int>(round_up(int64_t(cch) * t.Dt * 2, 16)) +
+                             static_cast<int>(round_up(cch * 4, 16));
+        if (win) t.stage_offs_bytes += cch * v.warps_dm * 4;
     }
     size_t p_bytes = 0;
     if (v.kind == 2 || v.kind == 4)  // 2 partial-sum slots, each with the chunk's trial offsets
@@ -338,6 +383,9 @@ dd_status build_fwd_tables(dd_plan_s *p, const dd_variant &v, FwdTables *out) {
         t.stage_offs_bytes += t.n_copies * 16;
         t.smem_bytes += size_t(v.stages) * t.n_copies * 16;
     }
+    if (win)  // the slots also hold every warp's output run while it is stored
+        t.smem_bytes = std::max(t.smem_bytes, 128 + size_t(v.warps_dm) * v.warps_time * 32 *
+                                                        v.samples_per_thread * 4);
     if (t.smem_bytes > p->smem_optin)
         return fail(DD_ERR_ARG, "variant needs more shared memory than the device has");
 
@@ -381,6 +429,9 @@ dd_status build_fwd_tables(dd_plan_s *p, const dd_variant &v, FwdTables *out) {
         e = upload(reinterpret_cast<void **>(&t.d_live), live.data(), live.size() * sizeof(int2));
     if (e == cudaSuccess)
         e = upload(reinterpret_cast<void **>(&t.d_offs), offs.data(), offs.size() * sizeof(uint16_t));
+    if (e == cudaSuccess && win)
+        e = upload(reinterpret_cast<void **>(&t.d_codes), codes.data(),
+                   codes.size() * sizeof(uint32_t));
     if (e == cudaSuccess && sb)
         e = upload(reinterpret_cast<void **>(&t.d_bdesc), bdesc.data(), bdesc.size() * sizeof(int4));
     if (e == cudaSuccess) e = cudaStreamSynchronize(t.aux);
@@ -396,25 +447,21 @@ dd_status build_fwd_tables(dd_plan_s *p, const dd_variant &v, FwdTables *out) {
 // make sure no launch still reads them (LaunchTracker::wait, or their own
 // synchronisation).
 void free_fwd_tables(FwdTables *t) {
-    void *ptrs[] = {t->d_copies, t->d_offs, t->d_bdesc, t->d_live};
+    void *ptrs[] = {t->d_copies, t->d_offs, t->d_bdesc, t->d_codes, t->d_live};
     for (void *q : ptrs)
         if (q) cudaFreeAsync(q, t->aux);
     t->d_copies = nullptr;
     t->d_offs = nullptr;
     t->d_bdesc = nullptr;
+    t->d_codes = nullptr;
     t->d_live = nullptr;
 }
 
 namespace {
 
-// Candidate default variants, best first; the first that fits the plan is
-// used until dd_tune or dd_plan_set_variant picks another.
-// (Measured on GB300: the wide sub-band kinds with 64-trial by 256-sample
-// tiles lead on the Apertif-like and 512-channel setups, kind 6 with 32
-// channels per stage first (2.34 against 2.43 ms for kind 4 with 16 at the
-// survey scale), then kind 2's 64 x 128 tiles; the lane-strided kind 0
-// takes setups whose delay patterns are too varied for sub-bands, e.g.
-// wide low-frequency bands.)
+// Variants tried in this order when none of the modelled candidates
+// (dd_default.cpp) fits a plan; the last ones fit every delay table that any
+// variant fits.
 const dd_variant kDefaults[] = {
     {6, 4, 8, 16, 1, 32, 2}, {4, 4, 8, 16, 1, 16, 2}, {2, 8, 4, 8, 1, 16, 2}, {2, 8, 4, 4, 2, 8, 2},
     {0, 4, 8, 4, 1, 8, 3},   {0, 4, 4, 4, 2, 8, 3},  {0, 4, 4, 4, 2, 4, 2},
@@ -512,21 +559,20 @@ dd_status finish_plan(dd_plan_s *p, dd_plan *out) {
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemset(err)");
 
     dd_status s = DD_ERR_UNSUPPORTED;
-    // 8- and 16-bit input: the wide sub-band CTAs fit 32 channels per stage
-    // (a quarter or half of the FP32 staging bytes), which halves the chunk
-    // barriers (measured on GB300 at the survey scale: 2.26 against 2.61 ms
-    // with 16 channels per stage for 8-bit input)
-    const dd_variant narrow_default = {4, 4, 8, 16, 1, 32, 2};
     dd_variant cached{};
     bool cached_tm = false;
     if (cache_lookup(plan_signature(p), &cached, &cached_tm)) {
         s = build_fwd_tables(p, cached, &p->fwd);
         if (s == DD_OK) p->fwd.time_major = cached_tm;
     }
-    if (s != DD_OK && p->dtype != DD_F32) {
-        s = build_fwd_tables(p, narrow_default, &p->fwd);
-        if (s != DD_OK && s != DD_ERR_ARG) return s;
-    }
+    if (s != DD_OK)
+        for (const RankedVariant &r : ranked_variants(p)) {
+            s = build_fwd_tables(p, r.v, &p->fwd);
+            if (s != DD_OK && s != DD_ERR_ARG) return s;
+            if (s != DD_OK) continue;
+            p->fwd.time_major = r.time_major;
+            break;
+        }
     for (size_t i = 0; s != DD_OK && i < sizeof(kDefaults) / sizeof(kDefaults[0]); ++i) {
         s = build_fwd_tables(p, kDefaults[i], &p->fwd);
         if (s != DD_OK && s != DD_ERR_ARG) return s;

@@ -25,7 +25,8 @@ namespace dd {
 dd_status sweep_variants(int32_t budget_ms, double flop,
                          const std::function<dd_status(const dd_variant &, double *)> &time_ms,
                          dd_variant *best, dd_tune_report *rep,
-                         const std::function<dd_status(const dd_variant &)> &between_passes) {
+                         const std::function<dd_status(const dd_variant &)> &between_passes,
+                         const std::vector<dd_variant> &extra) {
     const auto wall0 = std::chrono::steady_clock::now();
     auto over = [&]() {
         return budget_ms > 0 && std::chrono::duration<double, std::milli>(
@@ -54,6 +55,11 @@ dd_status sweep_variants(int32_t budget_ms, double flop,
         return DD_OK;
     };
     const int n = dd_variant_count();
+    for (const dd_variant &v : extra) {
+        if (over() && !tried.empty()) break;
+        dd_status s = run(v);
+        if (s != DD_OK) return s;
+    }
     // pass 1: every (kernel key, CTA shape) at the first staging choice of
     // the grid that fits the plan (8 channels per stage and 3 stages first;
     // a shape whose windows need smaller chunks, e.g. one staging a window
@@ -212,7 +218,9 @@ extern "C" dd_status dd_tune(dd_plan p, int32_t budget_ms, dd_tune_report *rep) 
     };
     const double flop = double(p->B) * p->D * double(p->S) * p->C;
     dd_variant best{};
-    dd_status s = sweep_variants(budget_ms, flop, time_ms, &best, rep, pick_order);
+    std::vector<dd_variant> extra;
+    for (const RankedVariant &r : ranked_variants(p)) extra.push_back(r.v);
+    dd_status s = sweep_variants(budget_ms, flop, time_ms, &best, rep, pick_order, extra);
     FwdTables t;
     if (s == DD_OK) s = build_fwd_tables(p, best, &t);
     if (s != DD_OK) {
