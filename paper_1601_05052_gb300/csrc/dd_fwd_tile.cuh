@@ -229,12 +229,13 @@ struct Stager {
                      in_b + (long long)(c0 + d.w) * a.stride + t0 + d.x, bytes, full);
     }
 
-    // Warp-cooperative: stage chunk k into `slot`. Lane l issues the chunk's
-    // copy l (at most 32 per chunk; `dsc` preloaded), lane 0 also the tables
-    // and weights. All 32 lanes of one warp must call it.
-    // `ahead`: chunk k + ahead's staging copies come with chunk k (0: none do).
+    // Warp-cooperative: announces chunk k's bytes on `full` and, if told so,
+    // issues its window copies (lane l copy l; at most 32 per chunk; `dsc`
+    // preloaded); lane 0 copies the tables and weights. All 32 lanes of one
+    // warp must call it. `ahead`: chunk k + ahead's staging copies come with
+    // chunk k (0: none do).
     __device__ __forceinline__ void issue(int k, int slot, int4 dsc, uint64_t *full, int lane,
-                                          int ahead = 0) const {
+                                          int ahead = 0, bool windows = true) const {
         unsigned char *sb = stage0 + slot * stage_bytes;
         const int c0 = (kc0 + k) * a.cch;
         const int nch = min(a.cch, a.C - c0);
@@ -248,7 +249,7 @@ struct Stager {
         if (lane == 0) mbar_arrive_expect_tx(full, total + tab_bytes + w_bytes + d_bytes);
         __syncwarp();
         fence_proxy_async_smem();
-        copy(sb, c0, dsc, full);
+        if (windows) copy(sb, c0, dsc, full);
         if (lane == 0) {
             unsigned char *tb = sb + a.stage_data_bytes;
             if (!subband) {
@@ -271,6 +272,30 @@ struct Stager {
             if (d_bytes)
                 bulk_g2s(tb + tab_bytes + weight_bytes(),
                          copies_k + (size_t)(kc0 + k + ahead) * a.n_copies, d_bytes, full);
+        }
+    }
+
+    // All warps of the CTA together: stage a tile's first chunks (n <= S of
+    // them, into slots `slot`, slot + 1, ... modulo S, which nothing reads or
+    // fills any more). Warp w issues copies w, w + n_warps, ... of every chunk;
+    // one warp per chunk also announces the bytes (a copy may complete before
+    // that: the barrier's phase still waits for the announcing arrival). One
+    // warp alone takes 30-60 clocks per copy, which nothing hides at a tile's
+    // start: 64 channels x 64 trials x 4096 samples, one tile per CTA, 7.5 ->
+    // 6.1 us a launch. (The register windows' registers leave no room for this
+    // form: 114.6 -> 116.9 us for 96 such beams; there warp 0 issues all.)
+    __device__ __forceinline__ void issue_first(int n, int slot, int S, uint64_t *full, int warp,
+                                                int n_warps, int lane, int ahead, int n_chunks) const {
+        const int m = warp + lane * n_warps;
+        fence_proxy_async_smem();
+        for (int k = 0; k < n; ++k) {
+            if (m < a.n_copies)
+                copy(stage0 + slot * stage_bytes, (kc0 + k) * a.cch,
+                     copies_k[(size_t)(kc0 + k) * a.n_copies + m], &full[slot]);
+            if (warp == k % n_warps)
+                issue(k, slot, desc(k, lane), &full[slot], lane,
+                      ahead && k + ahead < n_chunks ? ahead : 0, false);
+            if (++slot == S) slot = 0;
         }
     }
 };
@@ -586,7 +611,7 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs &a, int dtile, int ttile,
     const int n_chunks = kr.y - kr.x;
     const Stager<T> st = make_stager<T>(a, dtile, b, t0, stage0, false, kr.x);
 
-    // Staging: warp 0 issues the first S chunks; chunk kn >= S is issued by the
+    // Staging: all warps (windows: warp 0) issue the first S chunks; chunk kn >= S is issued by the
     // warps in turn, at the end of their chunk kn - S + 1, once every warp has
     // released chunk kn - S (one chunk of slack for slower warps). Issuing a
     // chunk's copies takes one warp 1-2 thousand clocks; with warp 0 issuing
@@ -601,12 +626,15 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs &a, int dtile, int ttile,
     int slot = int(kbase % S), turn = 0;
     uint32_t parity = (kbase / S) & 1u;
     // the slots' earlier chunks were released by every warp before this tile
-    if (warp == 0) {
-        const int pro = min(int(S), n_chunks);
-        for (int k = 0, sl = slot; k < pro; ++k) {
-            st.issue(k, sl, st.desc(k, lane), &full[sl], lane, ahead(k));
-            if (++sl == int(S)) sl = 0;
-        }
+    if constexpr (WIN) {
+        if (warp == 0)
+            for (int k = 0, sl = slot; k < min(int(S), n_chunks); ++k) {
+                st.issue(k, sl, st.desc(k, lane), &full[sl], lane, ahead(k));
+                if (++sl == int(S)) sl = 0;
+            }
+    } else {
+        st.issue_first(min(int(S), n_chunks), slot, int(S), full, warp, n_warps, lane,
+                       a.copies_ahead ? int(S) - 1 : 0, n_chunks);
     }
 
     Acc acc[DPT][SPT];
@@ -897,6 +925,9 @@ __device__ __forceinline__ void fwd_tile_sb(const FwdArgs &a, int dtile, int tti
     const uint32_t poffs_bytes = st.tab1_bytes;
     const int pslot_bytes = a.p_elems * int(sizeof(Acc)) + int(poffs_bytes);
     unsigned char *pslot0 = stage0 + S * st.stage_bytes;
+    // the slots' earlier chunks were released before this tile
+    st.issue_first(min(int(S), n_chunks), int(kbase % S), int(S), full, warp, nc + 1, lane, 0,
+                   n_chunks);
 
     if (warp == nc) {
         // ---------------- producer warp
@@ -910,18 +941,16 @@ __device__ __forceinline__ void fwd_tile_sb(const FwdArgs &a, int dtile, int tti
         int4 q[kDescAhead];
 #pragma unroll
         for (int j = 0; j < kDescAhead; ++j)
-            q[j] = j < n_chunks ? st.desc(j, lane) : make_int4(0, 0, 0, 0);
-        for (int k0 = 0; k0 < n_chunks; k0 += kDescAhead) {
+            q[j] = int(S) + j < n_chunks ? st.desc(int(S) + j, lane) : make_int4(0, 0, 0, 0);
+        for (int k0 = int(S); k0 < n_chunks; k0 += kDescAhead) {
 #pragma unroll
             for (int j = 0; j < kDescAhead; ++j) {
                 const int k = k0 + j;
                 if (k < n_chunks) {
                     const uint32_t kg = kbase + uint32_t(k);
                     const int slot = int(kg % S);
-                    bool ok = true;
-                    if (kg >= S)
-                        ok = mbar_wait_bounded(&empty[slot], ((kg / S) - 1u) & 1u, a.err,
-                                               kWaitBudgetNs, gave_up);
+                    const bool ok = mbar_wait_bounded(&empty[slot], ((kg / S) - 1u) & 1u, a.err,
+                                                      kWaitBudgetNs, gave_up);
                     if (__all_sync(0xffffffffu, ok)) st.issue(k, slot, q[j], &full[slot], lane);
                     q[j] = k + kDescAhead < n_chunks ? st.desc(k + kDescAhead, lane)
                                                      : make_int4(0, 0, 0, 0);
