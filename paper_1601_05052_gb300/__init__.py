@@ -28,12 +28,21 @@ def _lib_():
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    """The given or the current stream's handle. (torch.cuda.current_stream()
+    builds a Stream object: 3.1 us a call, against 0.2 us for the raw handle;
+    a 64-channel beam's whole call is about 10.)"""
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def compute_shifts(freqs, f_ref, t_samp, dms) -> np.ndarray:
