@@ -71,7 +71,8 @@ typedef struct dd_stream_s *dd_stream;
  * 32 * samples_per_thread * warps_time output samples; input rows of
  * chans_per_stage channels are staged per pipeline stage, `stages` deep.
  * kind 0: lane l of a warp owns samples l, l+32, ...; each add reads its
- *         input from shared memory.
+ *         input from shared memory. With 20 samples per thread (8-bit input
+ *         only) a lane owns consecutive samples and reads them as words.
  * kind 1: a thread owns samples_per_thread (odd) consecutive samples and
  *         keeps, per channel, the union window of its warp's trials in
  *         registers, serving every trial of the warp from it.
@@ -97,9 +98,10 @@ typedef struct {
     int32_t warps_dm;            /* warps along the DM axis of a CTA        */
     int32_t warps_time;          /* warps along the time axis of a CTA      */
     int32_t chans_per_stage;     /* channels per pipeline stage: 4, 8, 16, 32;
-                                  * 1 and 2 too for kind 0 with 8 x 8 outputs
-                                  * per thread and kind 5 with 14, 18 or 22
-                                  * samples, which may have 16 trial warps   */
+                                  * 1 and 2 too for kind 0 with 8 x 8 or 4 x 20
+                                  * outputs per thread and kind 5 with 14, 18
+                                  * or 22 samples, which may have 16 trial
+                                  * warps                                     */
     int32_t stages;              /* shared-memory pipeline depth (2..4)     */
 } dd_variant;
 

@@ -9,11 +9,11 @@
 // channel, G the staged words, cch the channels per stage. The tiles run in
 // rounds of the CTAs that are resident at once; staged bytes (L2) and
 // compulsory bytes (HBM) bound the sum from below. The constants of each
-// kernel family were fitted on a GB300 to timings of 204 setups drawn from
+// kernel family were fitted on a GB300 to timings of 272 setups drawn from
 // five bands (64-channel L-band, Apertif, 300 MHz L-band, 120-180 MHz, LOFAR;
 // 1 to 384 beams, 16 to 1024 channels, 4 to 2048 trials, all four input types),
-// each with every candidate that fits it (6500 in all). Residual 10 % (lane-strided,
-// windows) to 15 % (sub-bands, whose pattern count is not modelled). Over
+// each with every candidate that fits it. Residual 6 % (quads) and 10 %
+// (lane-strided, windows) to 15 % (sub-bands, whose patterns are not counted). Over
 // those setups the model's choice took 1.03 times the best candidate's time in
 // the geometric mean (1.31 at worst); the fixed preference list it replaced,
 // 1.39 times (5.2 at worst, LOFAR).
@@ -50,6 +50,12 @@ const Candidate kCandidates[] = {
     {{5, 4, 18, 4, 1, 8, 3}, false},
     {{5, 4, 14, 8, 1, 8, 3}, false},
     {{5, 4, 14, 4, 1, 8, 3}, false},
+    // byte quads: 8-bit input whose channel groups share few patterns
+    {{0, 4, 20, 4, 2, 16, 3}, false},
+    {{0, 4, 20, 8, 1, 16, 3}, false},
+    {{0, 4, 20, 4, 1, 16, 3}, false},
+    {{0, 4, 20, 2, 2, 16, 3}, false},
+    {{0, 4, 20, 1, 4, 4, 3}, true},
     // lane-strided: few trials, little work, or delays far apart
     {{0, 8, 8, 1, 8, 4, 3}, false},
     {{0, 8, 8, 2, 4, 8, 3}, false},
@@ -73,6 +79,7 @@ struct Fit {
     double a, b, k, l, o, s, m;
 };
 constexpr Fit kLane{0.95, 3.82, 1.55, 4.97, 6.49, 0, 13.84};
+constexpr Fit kQuad{1.3, 15.7, 2.84, 41.3, 6.12, 0, 7.05};
 constexpr Fit kWindow{1.21, 8.26, 0, 32.3, 9.1, 0, 8.41};
 constexpr Fit kReuse{0.58, 11.6, 11.2, 22.9, 3.93, 0, 34.8};
 constexpr Fit kSub2{1.03, 4.96, 0.73, 34.8, 1.84, 10.8, 3.44};
@@ -83,7 +90,8 @@ constexpr Fit kSub6{0.06, 9.76, 8.19, 24.1, 2.69, 148, 3.01};
 int registers(const dd_variant &v) {
     if (v.kind == 2) return v.dm_per_thread * v.samples_per_thread <= 16 ? 72 : 80;
     if (v.kind == 4 || v.kind == 6) return 96;
-    if (is_window(v.kind, v.samples_per_thread)) return 128;
+    if (is_window(v.kind, v.samples_per_thread) || is_quad(v.kind, v.samples_per_thread))
+        return 128;
     if (v.kind == 5) return 90;
     const int n = v.dm_per_thread * v.samples_per_thread;
     return n <= 8 ? 40 : (n <= 16 ? 56 : (n <= 32 ? 76 : 126));
@@ -112,7 +120,9 @@ DelaySteps delay_steps(const dd_plan_s *p) {
 // Modelled time of one forward launch in microseconds.
 double model_us(const dd_plan_s *p, const DelaySteps &st, const dd_variant &v) {
     const bool sb = is_subband(v.kind), win = is_window(v.kind, v.samples_per_thread);
-    const Fit &f = v.kind == 0   ? kLane
+    const bool quad = is_quad(v.kind, v.samples_per_thread);
+    const Fit &f = quad          ? kQuad
+                   : v.kind == 0 ? kLane
                    : win         ? kWindow
                    : v.kind == 5 ? kReuse
                    : v.kind == 2 ? kSub2
@@ -141,7 +151,9 @@ double model_us(const dd_plan_s *p, const DelaySteps &st, const dd_variant &v) {
     // evenly over [0, 2 mean], `same` of adjacent trials share a delay.
     const double x = 2 * st.mean, same = x <= 1 ? 1 - x / 2 : 1 / (2 * x);
     double W = v.dm_per_thread * v.samples_per_thread;
-    if (win && st.max <= kWinBands + 0.5)
+    if (quad)
+        W = v.dm_per_thread * (v.samples_per_thread / 4 + 1);
+    else if (win && st.max <= kWinBands + 0.5)
         W = 2 * (v.samples_per_thread / 2 + 3 * st.mean);
     else if (v.kind == 5 && !win)
         W *= 1 - same * (v.dm_per_thread - 1) / v.dm_per_thread;
@@ -164,6 +176,7 @@ std::vector<RankedVariant> ranked_variants(const dd_plan_s *p) {
     const DelaySteps st = delay_steps(p);
     std::vector<RankedVariant> r;
     for (const Candidate &c : kCandidates) {
+        if (is_quad(c.v.kind, c.v.samples_per_thread) && p->dtype != DD_U8) continue;
         // Windows want 32-bit samples (narrower ones at odd strides collide in
         // the banks: 64 channels x 64 trials, 8-bit, 22.6 against 9.4 us).
         if (is_window(c.v.kind, c.v.samples_per_thread) && p->dtype != DD_F32) continue;

@@ -116,7 +116,14 @@ const std::vector<FwdKernelKey> &fwd_compiled_keys() {
 }
 
 bool fwd_variant_compiled(int kind, int dpt, int spt) {
-    return pick_fwd(DD_F32, kind, dpt, spt, false).fn != nullptr;
+    return std::any_of(fwd_compiled_keys().begin(), fwd_compiled_keys().end(),
+                       [&](const FwdKernelKey &k) {
+                           return k.kind == kind && k.dpt == dpt && k.spt == spt;
+                       });
+}
+
+bool fwd_variant_has_type(dd_dtype t, int kind, int dpt, int spt) {
+    return pick_fwd(t, kind, dpt, spt, false).fn != nullptr;
 }
 
 dd_status launch_forward(dd_plan_s *p, const FwdTables &t, const void *in, const void *w,

@@ -60,9 +60,15 @@
     X(0, 2, 4) X(0, 4, 2) X(0, 4, 4) X(0, 8, 2) X(0, 8, 4) X(0, 4, 8) X(1, 8, 9) X(2, 4, 4) \
         X(2, 4, 8) X(2, 8, 4) X(2, 8, 2) X(3, 8, 4) X(3, 4, 8) X(3, 8, 2) X(4, 8, 4) X(4, 4, 8) \
             X(5, 4, 8) X(5, 8, 4) X(6, 4, 8) X(0, 4, 16) X(5, 4, 14) X(5, 4, 18) X(5, 4, 22) \
-                X(0, 8, 8)
+                X(0, 8, 8) X(0, 4, 20)
 
 namespace dd {
+
+// Whether a key has a kernel for an input type (the byte quads: 8-bit only).
+template <typename T>
+constexpr bool key_has_type(int kind, int spt) {
+    return !is_quad(kind, spt) || sizeof(T) == 1;
+}
 
 // Largest relative delay inside a warp's trial group served from registers.
 constexpr int kRwRmax = 15;
@@ -341,15 +347,18 @@ __device__ __forceinline__ void store_lane_strided(const FwdArgs &a, const Acc (
     }
 }
 
-// Stores a thread's accumulators of the register-window kernels: each warp
-// turns one trial at a time around in its own 32 * SPT words of shared memory
-// (the staging slots, which nothing reads any more once every warp has passed
-// the barrier), so that the lanes' stores to global memory are coalesced.
-template <typename Acc, int DPT, int SPT>
-__device__ __forceinline__ void store_window(const FwdArgs &a, const Acc (&acc)[DPT][SPT], int dtile,
-                                             int b, long long t0, int wd, int wt, int lane, int warp,
-                                             volatile int *gave_up, unsigned char *stage0) {
-    constexpr int M = SPT / 2;
+// Stores a thread's accumulators where it owns RUNS runs of consecutive
+// samples (register windows: 2, sample j of run r in acc[i][2 j + r]; byte
+// quads: 1): each warp turns one trial at a time around in its own 32 * SPT
+// words of shared memory (the staging slots, which nothing reads any more once
+// every warp has passed the barrier), so that the lanes' stores to global
+// memory are coalesced. (An odd run length keeps the turn free of conflicts;
+// the quads' 20 collide four ways, 0.3 % of their time at 256 channels.)
+template <int RUNS, typename Acc, int DPT, int SPT>
+__device__ __forceinline__ void store_runs(const FwdArgs &a, const Acc (&acc)[DPT][SPT], int dtile,
+                                           int b, long long t0, int wd, int wt, int lane, int warp,
+                                           volatile int *gave_up, unsigned char *stage0) {
+    constexpr int M = SPT / RUNS;
     __syncthreads();
     if (!*gave_up) {
         Acc *buf = reinterpret_cast<Acc *>(stage0) + warp * 32 * SPT;
@@ -358,10 +367,10 @@ __device__ __forceinline__ void store_window(const FwdArgs &a, const Acc (&acc)[
             const int d = dtile * a.Dt + wd * DPT + i;
             if (d >= a.D) break;
 #pragma unroll
-            for (int j = 0; j < M; ++j) {
-                buf[lane * M + j] = acc[i][2 * j];
-                buf[32 * M + lane * M + j] = acc[i][2 * j + 1];
-            }
+            for (int j = 0; j < M; ++j)
+#pragma unroll
+                for (int r = 0; r < RUNS; ++r)
+                    buf[32 * M * r + lane * M + j] = acc[i][RUNS * j + r];
             __syncwarp();
             Acc *orow = static_cast<Acc *>(a.out) + ((long long)b * a.D + d) * a.S + t0 +
                         wt * 32 * SPT + lane;
@@ -554,6 +563,90 @@ struct Window {
     }
 };
 
+// Byte quads (kind 0 with 20 samples per thread, 8-bit input). Lane l of a
+// warp owns M = 20 consecutive samples, M / 4 = 5 words apart from its
+// neighbours' (an odd number: the lanes' word loads are conflict-free), and
+// takes the channels two at a time. Per trial and channel it reads the M / 4 +
+// 1 words that hold its samples, 0.3 words per add where kind 0's byte loads
+// read one, shifts them by the delay's two low bits, interleaves the two
+// channels' bytes and adds both channels' products with one 16-bit by 8-bit
+// dot product per sample. Weights beyond 16 bits take byte extracts and
+// multiply-adds. Whole numbers: the sums are the same bits in any order. Bound
+// by issue slots (1.8 per add at 0.74 a clock; shared-memory pipe 51 %, integer
+// pipe 59 % busy). 32 beams x 256 channels over 120-180 MHz x 2000 trials x
+// 10000 samples: 17.8 ms (kind 0, 8 x 8) -> 10.2 ms; survey scale 2.65 against
+// the sub-bands' 2.25 ms. (Four channels at a time would halve the dot
+// products of weights below 256 but needs a byte transpose, as many integer
+// instructions more.)
+template <int SPT>
+struct Quads {
+    static constexpr int DPT = 4, Q = SPT / 4;
+
+    // acc += (wc.lo, wc.hi) . two bytes of b: bytes 0, 1 or bytes 2, 3
+    static __device__ __forceinline__ void dot_lo(int &acc, uint32_t wc, uint32_t b) {
+        asm("dp2a.lo.s32.u32 %0, %1, %2, %0;" : "+r"(acc) : "r"(wc), "r"(b));
+    }
+    static __device__ __forceinline__ void dot_hi(int &acc, uint32_t wc, uint32_t b) {
+        asm("dp2a.hi.s32.u32 %0, %1, %2, %0;" : "+r"(acc) : "r"(wc), "r"(b));
+    }
+    // the thread's samples of a channel for a trial at byte offset o
+    static __device__ __forceinline__ void words(uint32_t (&v)[Q], const uint8_t *sl, int o) {
+        const uint32_t *p = reinterpret_cast<const uint32_t *>(sl + (o & ~3));
+        const uint32_t sh = uint32_t(o) << 3;  // the funnel shift takes it modulo 32
+        uint32_t r[Q + 1];
+#pragma unroll
+        for (int k = 0; k <= Q; ++k) r[k] = p[k];
+#pragma unroll
+        for (int k = 0; k < Q; ++k) v[k] = __funnelshift_r(r[k], r[k + 1], sh);
+    }
+    // Two channels: offsets oa and ob, weights wa and wb (NARROW: both fit 16
+    // bits).
+    template <bool NARROW>
+    static __device__ __forceinline__ void channels(int (&acc)[DPT][SPT], const uint8_t *sl,
+                                                    const int (&oa)[DPT], const int (&ob)[DPT],
+                                                    int wa, int wb) {
+        const uint32_t wc = __byte_perm(uint32_t(wa), uint32_t(wb), 0x5410);
+#pragma unroll
+        for (int i = 0; i < DPT; ++i) {
+            uint32_t a[Q], b[Q];
+            words(a, sl, oa[i]);
+            words(b, sl, ob[i]);
+#pragma unroll
+            for (int k = 0; k < Q; ++k) {
+                if constexpr (NARROW) {
+                    const uint32_t lo = __byte_perm(a[k], b[k], 0x5140);
+                    const uint32_t hi = __byte_perm(a[k], b[k], 0x7362);
+                    dot_lo(acc[i][4 * k], wc, lo);
+                    dot_hi(acc[i][4 * k + 1], wc, lo);
+                    dot_lo(acc[i][4 * k + 2], wc, hi);
+                    dot_hi(acc[i][4 * k + 3], wc, hi);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        acc[i][4 * k + j] += wa * int(a[k] >> (8 * j) & 0xffu) +
+                                             wb * int(b[k] >> (8 * j) & 0xffu);
+                }
+            }
+        }
+    }
+
+    // A chunk's nch channels; `offs` the warp's trial offsets, Dt apart.
+    template <bool NARROW>
+    static __device__ __forceinline__ void chunk(int (&acc)[DPT][SPT], const uint8_t *sl,
+                                                 const uint16_t *offs, int Dt, const int *sw,
+                                                 int nch) {
+#pragma unroll 1
+        for (int cc = 0; cc < nch; cc += 2) {
+            // an odd last channel is paired with itself at weight 0
+            const int cb = min(cc + 1, nch - 1);
+            int oa[DPT], ob[DPT];
+            load_offsets<DPT>(offs + cc * Dt, oa);
+            load_offsets<DPT>(offs + cb * Dt, ob);
+            channels<NARROW>(acc, sl, oa, ob, sw[cc], cb > cc ? sw[cb] : 0);
+        }
+    }
+};
+
 // Barriers: every kind uses full[s] = bars[s] (producer arrival + bytes) and
 // empty[s] = bars[8 + s]: one arrival per warp for kinds 0/1, one per chunk
 // for kind 2 (after its compute barrier), one per builder warp for kind 3,
@@ -593,7 +686,7 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs &a, int dtile, int ttile,
         KIND == 1, RegWindow<T, DPT, SPT>, LaneStrided<T, DPT, SPT, KIND == 5>>::type;
     using Acc = typename Elem<T>::Acc;
     using Wt = typename Elem<T>::W;
-    constexpr bool WIN = is_window(KIND, SPT);
+    constexpr bool WIN = is_window(KIND, SPT), QUAD = is_quad(KIND, SPT);
     // With two slots, a refill at the end of a chunk leaves no copy in flight
     // during the next one; the kernels with the largest tiles, whose slots
     // leave no room for a third, refill before they sum a chunk (LOFAR, 8
@@ -642,7 +735,9 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs &a, int dtile, int ttile,
     for (int i = 0; i < DPT; ++i)
 #pragma unroll
         for (int j = 0; j < SPT; ++j) acc[i][j] = Acc(0);
-    const int lb = WIN ? wt * 32 * SPT + lane * (SPT / 2) : P::lane_base(wt, lane);
+    const int lb = WIN    ? wt * 32 * SPT + lane * (SPT / 2)
+                   : QUAD ? wt * 32 * SPT + lane * SPT
+                          : P::lane_base(wt, lane);
 
     // stages the chunk that goes into chunk k - 1's slot (sb: chunk k's slot)
     auto refill = [&](int k, const unsigned char *sb) {
@@ -692,6 +787,12 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs &a, int dtile, int ttile,
                 code = code_next;
                 wc = w_next;
             }
+        } else if constexpr (QUAD) {
+            const int wl = lane < nch ? sw[lane] : 0;  // nch <= 32
+            if (__all_sync(0xffffffffu, wl == int(short(wl))))
+                Quads<SPT>::template chunk<true>(acc, sdata + lb, soffs, a.Dt, sw, nch);
+            else
+                Quads<SPT>::template chunk<false>(acc, sdata + lb, soffs, a.Dt, sw, nch);
         } else {
             for (int cc = 0; cc < nch; ++cc) {
                 int o[DPT];
@@ -709,8 +810,9 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs &a, int dtile, int ttile,
         }
     }
     kbase += uint32_t(n_chunks);
-    if constexpr (WIN) {
-        store_window<Acc, DPT, SPT>(a, acc, dtile, b, t0, wd, wt, lane, warp, gave_up, stage0);
+    if constexpr (WIN || QUAD) {
+        store_runs<WIN ? 2 : 1, Acc, DPT, SPT>(a, acc, dtile, b, t0, wd, wt, lane, warp, gave_up,
+                                               stage0);
         return;
     }
     if (*gave_up) return;

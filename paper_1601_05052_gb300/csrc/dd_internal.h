@@ -176,10 +176,11 @@ dd_status cuda_fail(cudaError_t e, const char *what);
 dd_status ok();
 
 // Compiled forward variants: (kind, dm_per_thread, samples_per_thread) with a
-// kernel for every input type.
+// kernel for every input type (fwd_variant_has_type: some only for one).
 struct FwdKernelKey { int kind, dpt, spt; };
 const std::vector<FwdKernelKey> &fwd_compiled_keys();
 bool fwd_variant_compiled(int kind, int dpt, int spt);
+bool fwd_variant_has_type(dd_dtype t, int kind, int dpt, int spt);
 
 // Builds (or rebuilds) the forward tables for variant v; DD_ERR_ARG if v does
 // not fit this plan/device.

@@ -113,7 +113,8 @@ int occupancy_t(int block, size_t smem) {
 template <typename T, bool LIVE>
 FwdKernel pick(int kind, int dpt, int spt) {
 #define DD_PICK(K_, D_, S_)                                                   \
-    if (kind == K_ && dpt == D_ && spt == S_)                                 \
+    if constexpr (key_has_type<T>(K_, S_))                                    \
+        if (kind == K_ && dpt == D_ && spt == S_)                             \
         return FwdKernel{(const void *)&dd_fwd_kernel<K_, T, D_, S_, LIVE>,   \
                          &launch_fwd_t<K_, T, D_, S_, LIVE>};
     DD_FWD_KEYS(DD_PICK)
@@ -125,7 +126,8 @@ FwdKernel pick(int kind, int dpt, int spt) {
 template <typename T>
 PersistentFn pick_persistent(int kind, int dpt, int spt) {
 #define DD_PICK(K_, D_, S_)                                                         \
-    if (kind == K_ && dpt == D_ && spt == S_)                                       \
+    if constexpr (key_has_type<T>(K_, S_))                                          \
+        if (kind == K_ && dpt == D_ && spt == S_)                                   \
         return PersistentFn{(const void *)&dd_fwd_persistent_kernel<K_, T, D_, S_>, \
                             &occupancy_t<K_, T, D_, S_>};
     DD_FWD_KEYS(DD_PICK)

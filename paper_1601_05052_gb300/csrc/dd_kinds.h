@@ -30,10 +30,13 @@ __host__ __device__ constexpr bool is_subband(int kind) {
 __host__ __device__ constexpr bool is_window(int kind, int spt) {
     return kind == 5 && spt % 4 == 2;
 }
+// Byte-quad form of kind 0 (8-bit input only): 20 consecutive samples per
+// thread, read as 32-bit words.
+__host__ __device__ constexpr bool is_quad(int kind, int spt) { return kind == 0 && spt == 20; }
 // Kernels whose CTAs may have 16 trial warps and stage 1 or 2 channels at a time:
-// the register windows and the lane-strided 8 x 8 form.
+// the register windows, the byte quads and the lane-strided 8 x 8 form.
 __host__ __device__ constexpr bool is_wide(int kind, int dpt, int spt) {
-    return is_window(kind, spt) || (kind == 0 && dpt == 8 && spt == 8);
+    return is_window(kind, spt) || is_quad(kind, spt) || (kind == 0 && dpt == 8 && spt == 8);
 }
 // Codes of the delay steps a register window serves: steps (s1, s2, s3)
 // between a thread's four trials with every step in {b, b + 1} are code 7 b +

@@ -168,6 +168,8 @@ uint32_t window_code(const uint16_t *o, int n) {
 dd_status build_fwd_tables(dd_plan_s *p, const dd_variant &v, FwdTables *out) {
     dd_status s = check_variant_shape(v);
     if (s != DD_OK) return s;
+    if (!fwd_variant_has_type(p->dtype, v.kind, v.dm_per_thread, v.samples_per_thread))
+        return fail(DD_ERR_ARG, "variant not compiled for this input type");
     FwdTables t;
     t.v = v;
     t.Dt = v.dm_per_thread * v.warps_dm;
@@ -383,7 +385,7 @@ dd_status build_fwd_tables(dd_plan_s *p, const dd_variant &v, FwdTables *out) {
         t.stage_offs_bytes += t.n_copies * 16;
         t.smem_bytes += size_t(v.stages) * t.n_copies * 16;
     }
-    if (win)  // the slots also hold every warp's output run while it is stored
+    if (win || is_quad(v.kind, v.samples_per_thread))  // the slots also turn the outputs around
         t.smem_bytes = std::max(t.smem_bytes, 128 + size_t(v.warps_dm) * v.warps_time * 32 *
                                                         v.samples_per_thread * 4);
     if (t.smem_bytes > p->smem_optin)

@@ -113,6 +113,46 @@ def test_wide_lane_strided_equals_the_general_kernel(dtype, step):
     plan.check_device()
 
 
+@pytest.mark.parametrize("wkind", ["q8", "wide", "signed16"])
+@pytest.mark.parametrize("D,S,C", [(1, 1, 1), (5, 641, 7), (18, 1283, 12), (33, 640, 5)])
+def test_byte_quads_equal_the_general_kernel(D, S, C, wkind):
+    """20 consecutive 8-bit samples per thread: every delay modulo 4, odd
+    channel counts and chunks, weights within and beyond 16 bits (both ends),
+    extreme samples, few and many trials; a 32-bit plan refuses the variant."""
+    rng = np.random.default_rng(D * S + C)
+    sh = (np.arange(D)[:, None] * rng.integers(0, 23, C)[None, :]
+          + rng.integers(0, 8, (D, C))).astype(np.int64)
+    x, w = _inputs(sh, S, 2, "u8", rng)
+    x[:, 0] = 255
+    x[:, -1, ::3] = 0
+    if wkind == "signed16":
+        w = rng.integers(-32768, 32768, C).astype(np.int32)
+        w[0], w[-1] = -32768, 32767
+    elif wkind == "wide":
+        w = rng.integers(-(1 << 19), 1 << 19, C).astype(np.int32)
+        w[C // 2] = 40000
+    plan = Plan(shifts=sh, n_out=S, batch=2, dtype="u8")
+    xd, wd = to_dev(x, "u8"), weights_dev(w, "u8")
+    ref = oracle.forward_u8(x, w, sh, S)
+    ran = 0
+    for wd_, wt, cch, st in ((1, 8, 8, 3), (2, 4, 8, 2), (8, 1, 4, 4), (16, 1, 32, 2), (2, 1, 1, 2),
+                             (2, 2, 2, 3), (3, 1, 16, 3)):
+        plan.variant = _variant(0, 4, 20, wd_, wt, cch, st)
+        out = torch.full(plan.out_shape, 77, dtype=torch.int32, device="cuda")
+        np.testing.assert_array_equal(plan.execute(xd, wd, out).cpu().numpy(), ref,
+                                      err_msg=str(plan.variant))
+        ran += 1
+    assert ran == 7
+    batch = Batch([plan, plan])
+    batch.variant = _variant(0, 4, 20, 2, 2, 4, 2)
+    for out in batch.execute([xd, xd], [wd, wd]):
+        np.testing.assert_array_equal(out.cpu().numpy(), ref)
+    other = Plan(shifts=sh, n_out=S, batch=2)
+    with pytest.raises(DDError):
+        other.variant = _variant(0, 4, 20, 2, 2, 4, 2)
+    plan.check_device()
+
+
 def test_windows_in_a_batch_and_refused_shapes():
     """Two plans with different channel and trial counts in one persistent
     launch of the window kernel, twice; shapes that cannot be staged on
