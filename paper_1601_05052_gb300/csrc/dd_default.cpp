@@ -183,12 +183,16 @@ std::vector<RankedVariant> ranked_variants(const dd_plan_s *p) {
         // One partial-sum slot only where two do not fit (survey scale, 8-bit:
         // kind 4 2.26 ms, kind 6 2.38; FP32 fits 32 channels in kind 6 alone).
         if (c.v.kind == 6 && c.v.warps_dm == 16 && p->dtype != DD_F32) continue;
-        // Where no channel moves by more than half a sample per trial, a
+        // Where no channel moves by more than 0.8 samples per trial, a
         // thread's trials mostly share a sub-band's series and offset, which
         // the model does not see (500 channels x 1000 trials x 10000 samples,
         // FP32: sub-bands 0.51 ms, windows 0.59, lane-strided 1.2).
-        if (st.max <= 0.5 && p->D >= 24 && !is_subband(c.v.kind)) continue;
-        r.push_back(RankedVariant{c.v, c.time_major, model_us(p, st, c.v)});
+        if (st.max <= 0.8 && p->D >= 24 && !is_subband(c.v.kind)) continue;
+        // Near ties go to the wide sub-bands, whose grouped sums are also the
+        // more accurate (500 channels x 1000 trials, FP32: 0.54 ms where the
+        // model has 0.61, windows 0.615 where it has 0.56).
+        const double tie = is_subband(c.v.kind) && c.v.warps_dm == 16 ? 1.0 : 1.04;
+        r.push_back(RankedVariant{c.v, c.time_major, tie * model_us(p, st, c.v)});
     }
     std::stable_sort(r.begin(), r.end(),
                      [](const RankedVariant &a, const RankedVariant &b) { return a.us < b.us; });

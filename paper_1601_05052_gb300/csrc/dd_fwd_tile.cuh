@@ -178,6 +178,20 @@ __device__ __forceinline__ void compute_barrier(int n) {
     asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory");
 }
 
+// The same barrier, returning whether any of the threads came with `p` set.
+__device__ __forceinline__ bool compute_barrier_or(int n, bool p) {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred a, b;\n\t"
+        "setp.ne.u32 a, %1, 0;\n\t"
+        "bar.red.or.pred b, 1, %2, a;\n\t"
+        "selp.u32 %0, 1, 0, b;\n\t}"
+        : "=r"(r)
+        : "r"(uint32_t(p)), "r"(n)
+        : "memory");
+    return r != 0;
+}
+
 // Packed FP32 pair arithmetic of sm_100-class GPUs (one instruction for two
 // lanes' worth of adds / fmas, each rounded to nearest like the scalar
 // forms): a += b and d = a * b + d element-wise.
@@ -1072,19 +1086,25 @@ __device__ __forceinline__ void fwd_tile_sb(const FwdArgs &a, int dtile, int tti
         for (int j = 0; j < SPT; ++j) acc[i][j] = Acc(0);
     const int lb = wt * 32 * SPT + lane;
 
+    // Slot and phase of a chunk are counted on (a division by the run-time
+    // number of slots takes about 150 clocks, which every warp waits for), and
+    // a lost wait travels with the barrier instead of being read from shared
+    // memory after it. Survey scale: FP32 (kind 6) 2.328 -> 2.280 ms, 8-bit
+    // 2.250 -> 2.232 ms. (16-bit input with two slots is the exception: 0.507
+    // ms with the flag, 0.536 with the barrier's answer, at 2 beams x 509
+    // channels x 777 trials x 10001 samples.)
+    uint32_t slot = kbase % S, parity = (kbase / S) & 1u;
     for (int k = 0; k < n_chunks; ++k) {
-        const uint32_t kg = kbase + uint32_t(k);
-        const int slot = int(kg % S);
-        // A failed wait sets the give-up flag before the barrier; after it
-        // every warp sees the flag and skips the trials on the chunk.
+        // A failed wait in any warp is known to all of them after the barrier;
+        // the chunk's trials are then skipped.
         const bool ok = __all_sync(
-            0xffffffffu,
-            mbar_wait_bounded(&full[slot], (kg / S) & 1u, a.err, kWaitBudgetNs, gave_up));
+            0xffffffffu, mbar_wait_bounded(&full[slot], parity, a.err, kWaitBudgetNs, gave_up));
         const unsigned char *sb = stage0 + slot * st.stage_bytes;
         const T *raw = reinterpret_cast<const T *>(sb);
         const int4 *bd = reinterpret_cast<const int4 *>(sb + a.stage_data_bytes + poffs_bytes);
         const Wt *sw = reinterpret_cast<const Wt *>(sb + a.stage_data_bytes + st.tab_bytes);
-        unsigned char *pb = pslot0 + (ONE_SLOT ? 0u : (kg & 1u)) * pslot_bytes;
+        unsigned char *pb =
+            pslot0 + (ONE_SLOT ? 0u : ((kbase + uint32_t(k)) & 1u)) * pslot_bytes;
         Acc *P = reinterpret_cast<Acc *>(pb);
         uint16_t *poffs = reinterpret_cast<uint16_t *>(pb + a.p_elems * int(sizeof(Acc)));
         const int ng = (min(a.cch, a.C - (kr.x + k) * a.cch) + kSbG - 1) / kSbG;
@@ -1096,19 +1116,27 @@ __device__ __forceinline__ void fwd_tile_sb(const FwdArgs &a, int dtile, int tti
             uint32_t *dst = reinterpret_cast<uint32_t *>(poffs);
             for (int i = tid; i < int(poffs_bytes / 4); i += nc * 32) dst[i] = src[i];
         }
-        compute_barrier(nc * 32);
+        bool lost;
+        if constexpr (sizeof(T) == 2 && !ONE_SLOT) {
+            compute_barrier(nc * 32);
+            lost = *gave_up;
+        } else {
+            lost = compute_barrier_or(nc * 32, !ok);
+        }
+        // nothing reads this staging slot any more (a lost chunk's is not
+        // released: the producer's next wait fails too)
+        if (tid == 0 && !lost) mbar_arrive(&empty[slot]);
+        if (++slot == S) {
+            slot = 0;
+            parity ^= 1u;
+        }
         if constexpr (ONE_SLOT) {
-            // every warp reaches both barriers of a chunk, whatever the flag
-            // (the producer may set it between two warps' reads)
-            if (!*gave_up) {
-                if (tid == 0) mbar_arrive(&empty[slot]);
+            if (!lost)
                 sb_trials<sb_passes<T, true>(), Acc, DPT, SPT>(acc, P + lb, poffs + wd * DPT, a.Dt,
                                                                ng);
-            }
             compute_barrier(nc * 32);
         } else {
-            if (*gave_up) continue;  // no arrival: the producer's next wait fails too
-            if (tid == 0) mbar_arrive(&empty[slot]);  // nothing reads this staging slot any more
+            if (lost) continue;
             sb_trials<sb_passes<T, false>(), Acc, DPT, SPT>(acc, P + lb, poffs + wd * DPT, a.Dt,
                                                             ng);
         }
