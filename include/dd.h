@@ -155,7 +155,8 @@ int32_t dd_plan_max_shift(dd_plan plan);
 /* Copies the delay table, int32 [n_dm][n_chan], to host memory. */
 dd_status dd_plan_shifts(dd_plan plan, int32_t *host_dst);
 
-/* Variant used by dd_execute. set: DD_ERR_ARG if the variant is not in the
+/* Variant used by dd_execute (a new plan starts with the tuning cache's, see
+ * dd_tune, or the one whose modelled time is smallest). set: DD_ERR_ARG if the variant is not in the
  * compiled grid or does not fit the device's shared memory for this plan;
  * before it frees the old tables it waits (on the host) for this plan's
  * earlier launches on every stream they went to, not for the whole device.
@@ -163,7 +164,7 @@ dd_status dd_plan_shifts(dd_plan plan, int32_t *host_dst);
  * are kept until the plan is destroyed (the graph may still replay them). */
 dd_status dd_plan_get_variant(dd_plan plan, dd_variant *v);
 dd_status dd_plan_set_variant(dd_plan plan, const dd_variant *v);
-/* Launch order of the forward kernel's tiles: DM tiles fastest (the default;
+/* Launch order of the forward kernel's tiles: DM tiles fastest (the usual one;
  * resident CTAs share a time range, so windows that neighbouring DM tiles
  * share stay in L2) or time tiles fastest (resident CTAs sweep one DM tile's
  * rows; better where neighbouring DM tiles read far-apart windows, e.g. the
@@ -248,7 +249,7 @@ dd_status dd_grad_w_noalloc(dd_plan plan, const float *d_gout, const float *d_in
  * creation (dd_plan_create, dd_plan_create_from_shifts) then starts from the
  * last line whose key matches, so the sweep is an offline step, as the paper
  * treats it. A missing or unreadable file, or a recorded variant that no
- * longer fits, falls back to the built-in defaults silently. */
+ * longer fits, falls back to the modelled default silently. */
 dd_status dd_tune(dd_plan plan, int32_t budget_ms, dd_tune_report *rep);
 
 /* Tunes the kernel variant of the adjoint's transposed dedispersion (the
@@ -278,7 +279,9 @@ dd_status dd_adjoint_set_variant(dd_plan plan, const dd_variant *v);
  * heaviest setup first. One launch runs one compiled kernel: all plans share
  * kind, dm_per_thread, samples_per_thread, stages and the number of trial
  * warps (warps_dm * warps_time); each plan has its own split of those warps
- * (its DM x time tile) and its own chans_per_stage. */
+ * (its DM x time tile) and its own chans_per_stage. A batch starts with the
+ * first plan's variant if that was set or tuned and fits every plan, else with
+ * the variant whose modelled time over all plans is smallest. */
 dd_status dd_batch_create(dd_batch *out, int32_t n, const dd_plan *plans);
 dd_status dd_batch_execute(dd_batch batch, const void *const *d_in,
                            const void *const *d_w, void *const *d_out, void *stream);

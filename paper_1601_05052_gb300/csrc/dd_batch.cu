@@ -291,9 +291,10 @@ dd_status dd_batch_create(dd_batch *out, int32_t n, const dd_plan *plans) {
         dd_batch_destroy(bt);
         return cuda_fail(e, "cudaMalloc(batch)");
     }
-    // The common variant with the smallest modelled time over all plans, among
+    // The first plan's variant if it was set or tuned and fits every plan; else
+    // the common variant with the smallest modelled time over all plans, among
     // those that fit every plan; else any compiled variant that does.
-    dd_status s = DD_ERR_ARG;
+    dd_status s = plans[0]->chosen ? configure(bt, plans[0]->fwd.v) : DD_ERR_ARG;
     const std::vector<RankedVariant> common = common_variants(bt->plans);
     for (size_t i = 0; i < common.size() && s != DD_OK; ++i) s = configure(bt, common[i].v);
     if (s != DD_OK) {

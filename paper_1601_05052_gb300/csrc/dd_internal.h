@@ -149,6 +149,7 @@ struct dd_plan_s {
     size_t smem_optin = 0;
 
     dd::FwdTables fwd;
+    bool chosen = false;  // fwd's variant was set, tuned or restored, not modelled
     dd::AdjState adj;
     int32_t *d_shifts = nullptr;  // device copy of `shifts`
     int *d_err = nullptr;         // device error word (dd::kErr* bits)

@@ -566,6 +566,7 @@ dd_status finish_plan(dd_plan_s *p, dd_plan *out) {
     if (cache_lookup(plan_signature(p), &cached, &cached_tm)) {
         s = build_fwd_tables(p, cached, &p->fwd);
         if (s == DD_OK) p->fwd.time_major = cached_tm;
+        p->chosen = s == DD_OK;
     }
     if (s != DD_OK)
         for (const RankedVariant &r : ranked_variants(p)) {
@@ -718,6 +719,7 @@ dd_status dd_plan_set_variant(dd_plan p, const dd_variant *v) {
     FwdTables t;
     dd_status s = build_fwd_tables(p, *v, &t);
     if (s != DD_OK) return s;
+    p->chosen = true;
     return replace_fwd_tables(p, &p->fwd, t);  // waits for this plan's launches only
 }
 

@@ -248,6 +248,7 @@ extern "C" dd_status dd_tune(dd_plan p, int32_t budget_ms, dd_tune_report *rep) 
     }
     s = replace_fwd_tables(p, &p->fwd, t);
     if (s != DD_OK) return s;
+    p->chosen = true;
     cache_store(plan_signature(p), best, t.time_major);
     return DD_OK;
 }
