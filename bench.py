@@ -46,6 +46,7 @@ METRIC = "DM-trial·samples/s"
 # profiles/ is only reported while they are unchanged.
 KERNEL_SOURCES = ["paper_1601_05052_gb300/csrc/dd_fwd_tile.cuh",
                   "paper_1601_05052_gb300/csrc/dd_fwd.cu",
+                  "paper_1601_05052_gb300/csrc/dd_kernels.cu",
                   "paper_1601_05052_gb300/csrc/dd_ptx.cuh",
                   "paper_1601_05052_gb300/csrc/dd_plan.cpp",
                   "paper_1601_05052_gb300/csrc/dd_kinds.h"]

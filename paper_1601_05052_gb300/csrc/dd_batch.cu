@@ -12,7 +12,8 @@
 // one block size and staging depth, but each plan has its own tile shape
 // within it: its split of the trial warps along DM and time (so its DM x
 // time tile) and its channels per stage, with its own staging tables; the
-// batch tuner picks the common kernel first and then each plan's shape. A
+// batch starts with the common variant of the smallest modelled time, and its
+// tuner picks the common kernel first and then each plan's shape. A
 // CTA finishes a tile (every chunk consumed) before it takes the next item,
 // so tiles of plans with different slot layouts never overlap in shared
 // memory, and the common staging depth keeps the mbarrier phases of

@@ -1,4 +1,4 @@
-// dd_fwd.cu -- forward dedispersion kernel for sm_103a and its launcher.
+// dd_fwd.cu -- launches of the forward dedispersion kernels (dd_kernels.cu).
 //
 // Computes out[b][d][t] = sum_c w[c] * in[b][c][t + shift[d][c]] (Algorithm
 // 1, Section III-A, with weights) with one CTA per (DM tile, time tile,
@@ -6,7 +6,7 @@
 // fastest along grid x, so that CTAs resident at the same time share time
 // ranges and the input windows they stage stay in L2. Where neighbouring DM
 // tiles read far-apart windows (delays that grow by more than a time tile
-// per trial), the tuner can take the time tile fastest instead: resident
+// per trial), the default or the tuner can take the time tile fastest: resident
 // CTAs then sweep one DM tile's rows, and the next DM tile, whose windows
 // are shifted by a few DM steps, finds them still in L2.
 #include <algorithm>

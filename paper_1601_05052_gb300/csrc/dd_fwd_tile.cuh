@@ -1,6 +1,5 @@
 // dd_fwd_tile.cuh -- the per-tile body of the forward dedispersion kernel,
-// shared by the one-shot launch (dd_fwd.cu) and the persistent batched
-// launch (dd_batch.cu).
+// shared by the one-shot and the persistent batched kernels (dd_kernels.cu).
 //
 // A tile is (beam b, DM tile of Dt trials, time tile of Ts output samples)
 // and computes out[b][d][t] = sum_c w[c] * in[b][c][t + shift[d][c]] for its
@@ -10,16 +9,19 @@
 // registers.
 //
 // Staging (Section III-B's shared "local memory"): channels are taken in
-// chunks. For each chunk one warp copies, per channel (one lane each), the
-// union of the tile's shifted input windows with a 1-D TMA bulk copy into a
-// pipeline slot, together with the chunk's tables and weights; the slot's
-// `full` mbarrier counts the bytes. Channel descriptors are read one chunk
-// ahead so the copies go out without waiting on global memory.
+// chunks. Per chunk the tile's shifted input windows are copied, one 1-D TMA
+// bulk copy per lane, into a pipeline slot, together with the chunk's tables
+// and weights; the slot's `full` mbarrier counts the bytes. A tile's first
+// chunks are issued by all warps together, later ones by one warp each: the
+// trial warps in turn (kinds 0, 1 and 5) or a producer or builder warp
+// (sub-bands). Copy lists are read ahead, so the copies go out without waiting
+// on global memory.
 //
 // Ways to turn a staged window into sums (the `kind` of a variant):
 //  kind 0, lane-strided: lane l owns samples l, l+32, ...; every add reads
 //    its operand from shared memory (conflict-free, one word per add).
 //    Slots are recycled through `empty` mbarriers (one arrival per warp).
+//    8-bit input with 20 samples per thread reads words (see Quads).
 //  kind 1, register window: a thread owns SPT (odd) consecutive samples;
 //    per channel it loads its warp's union window into registers once and
 //    serves every trial from it through a warp-uniform switch on the
