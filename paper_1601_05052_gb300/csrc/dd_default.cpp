@@ -186,8 +186,16 @@ std::vector<RankedVariant> ranked_variants(const dd_plan_s *p) {
         // Where no channel moves by more than 0.8 samples per trial, a
         // thread's trials mostly share a sub-band's series and offset, which
         // the model does not see (500 channels x 1000 trials x 10000 samples,
-        // FP32: sub-bands 0.51 ms, windows 0.59, lane-strided 1.2).
-        if (st.max <= 0.8 && p->D >= 24 && !is_subband(c.v.kind)) continue;
+        // FP32: sub-bands 0.51 ms, windows 0.59, lane-strided 1.2). And a
+        // float chain over more than 128 channels rounds more than the
+        // sub-bands' groups of four, so smooth delays keep those: 473 channels
+        // x 788 trials x 4406 samples, gradients, 5.2e-7 of the largest output
+        // against 2.8e-7, and 0.69 ms against 0.55. (Adjoints reach 26 samples
+        // per step at survey bands; low bands, at 39, leave the sub-bands
+        // nothing to share.)
+        if (p->D >= 24 && !is_subband(c.v.kind) &&
+            (st.max <= 0.8 || (p->dtype != DD_U8 && p->C > 128 && st.max <= 32)))
+            continue;
         // Near ties go to the wide sub-bands, whose grouped sums are also the
         // more accurate (500 channels x 1000 trials, FP32: 0.54 ms where the
         // model has 0.61, windows 0.615 where it has 0.56).
