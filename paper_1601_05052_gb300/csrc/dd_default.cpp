@@ -172,6 +172,17 @@ double model_us(const dd_plan_s *p, const DelaySteps &st, const dd_variant &v) {
     return us;
 }
 
+// Long float chains whose delays move by 12 to 32 samples per trial (adjoints
+// at survey bands; low bands start at 39): sub-bands round less there too, but
+// the model does not order them well enough (gradients of 3 x 268 channels x
+// 1886 trials x 10382 samples: its choice 5.8 ms, the preference list's 4.5;
+// windows 3.6 at twice the error).
+bool by_preference(const dd_plan_s *p) {
+    if (p->dtype == DD_U8 || p->C <= 128 || p->D < 24) return false;
+    const double steps = delay_steps(p).max;
+    return steps > 12 && steps <= 32;
+}
+
 std::vector<RankedVariant> ranked_variants(const dd_plan_s *p) {
     const DelaySteps st = delay_steps(p);
     std::vector<RankedVariant> r;
@@ -190,11 +201,9 @@ std::vector<RankedVariant> ranked_variants(const dd_plan_s *p) {
         // float chain over more than 128 channels rounds more than the
         // sub-bands' groups of four, so smooth delays keep those: 473 channels
         // x 788 trials x 4406 samples, gradients, 5.2e-7 of the largest output
-        // against 2.8e-7, and 0.69 ms against 0.55. (Adjoints reach 26 samples
-        // per step at survey bands; low bands, at 39, leave the sub-bands
-        // nothing to share.)
+        // against 2.8e-7, and 0.69 ms against 0.55.
         if (p->D >= 24 && !is_subband(c.v.kind) &&
-            (st.max <= 0.8 || (p->dtype != DD_U8 && p->C > 128 && st.max <= 32)))
+            (st.max <= 0.8 || (p->dtype != DD_U8 && p->C > 128 && st.max <= 12)))
             continue;
         // Near ties go to the wide sub-bands, whose grouped sums are also the
         // more accurate (500 channels x 1000 trials, FP32: 0.54 ms where the

@@ -568,7 +568,7 @@ dd_status finish_plan(dd_plan_s *p, dd_plan *out) {
         if (s == DD_OK) p->fwd.time_major = cached_tm;
         p->chosen = s == DD_OK;
     }
-    if (s != DD_OK)
+    if (s != DD_OK && !by_preference(p))
         for (const RankedVariant &r : ranked_variants(p)) {
             s = build_fwd_tables(p, r.v, &p->fwd);
             if (s != DD_OK && s != DD_ERR_ARG) return s;
