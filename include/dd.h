@@ -71,7 +71,9 @@ typedef struct dd_stream_s *dd_stream;
  * 32 * samples_per_thread * warps_time output samples; input rows of
  * chans_per_stage channels are staged per pipeline stage, `stages` deep.
  * kind 0: lane l of a warp owns samples l, l+32, ...; each add reads its
- *         input from shared memory. With 20 samples per thread (8-bit input
+ *         input from shared memory. With 2 x 4, 4 x 2 or 4 x 8 outputs per
+ *         thread, float sums take four channels at a time, as kind 2's do.
+ *         With 20 samples per thread (8-bit input
  *         only) a lane owns consecutive samples and reads them as words.
  * kind 1: a thread owns samples_per_thread (odd) consecutive samples and
  *         keeps, per channel, the union window of its warp's trials in

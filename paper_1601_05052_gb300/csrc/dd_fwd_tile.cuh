@@ -21,6 +21,7 @@
 //  kind 0, lane-strided: lane l owns samples l, l+32, ...; every add reads
 //    its operand from shared memory (conflict-free, one word per add).
 //    Slots are recycled through `empty` mbarriers (one arrival per warp).
+//    Three float forms sum groups of four channels first (see GroupedLanes).
 //    8-bit input with 20 samples per thread reads words (see Quads).
 //  kind 1, register window: a thread owns SPT (odd) consecutive samples;
 //    per channel it loads its warp's union window into registers once and
@@ -440,6 +441,69 @@ struct LaneStrided {
     }
 };
 
+// Grouped sums (float input, 2 x 4, 4 x 2 and 4 x 8 outputs per thread): four
+// channels' products of an output are summed first and then added to its
+// accumulator, a sub-band kernel's operations in the same order, so that both
+// give the same bits and a plan may take either. The reads stay one shared word
+// per add, which bounds the loop as before; 0.98-1.03 times the single chain's
+// time over 27 setups of 4 to 101 trials (384 beams x 64 channels x 4 trials x
+// 4096 samples, FP32: 72.9 -> 72.0 us, largest error 1.7e-7 -> 8.2e-8 of the
+// largest output; one beam, 64 trials: unchanged).
+template <typename T, int DPT, int SPT>
+struct GroupedLanes {
+    static constexpr int U = DPT * SPT > 8 ? 1 : 2;  // groups with their loads in flight at once
+
+    // A chunk's nch channels; `offs` the warp's trial offsets, Dt apart.
+    static __device__ __forceinline__ void chunk(float (&acc)[DPT][SPT], const T *s,
+                                                 const uint16_t *offs, int Dt, const float *sw,
+                                                 int nch) {
+        int cc = 0;
+#pragma unroll U
+        for (; cc + kSbG <= nch; cc += kSbG) {
+            const float4 w = *reinterpret_cast<const float4 *>(sw + cc);
+            int o[kSbG][DPT];
+#pragma unroll
+            for (int q = 0; q < kSbG; ++q) load_offsets<DPT>(offs + (cc + q) * Dt, o[q]);
+#pragma unroll
+            for (int i = 0; i < DPT; ++i) {
+                float v[SPT];
+#pragma unroll
+                for (int j = 0; j < SPT; ++j)
+                    v[j] = __fmul_rn(w.x, Elem<T>::val(s[o[0][i] + 32 * j]));
+#pragma unroll
+                for (int q = 1; q < kSbG; ++q) {
+                    const float wq = q == 1 ? w.y : (q == 2 ? w.z : w.w);
+                    const T *t = s + o[q][i];
+#pragma unroll
+                    for (int j = 0; j < SPT; j += 2)
+                        fma2(v[j], v[j + 1], wq, wq, Elem<T>::val(t[32 * j]),
+                             Elem<T>::val(t[32 * j + 32]));
+                }
+#pragma unroll
+                for (int j = 0; j < SPT; j += 2) add2(acc[i][j], acc[i][j + 1], v[j], v[j + 1]);
+            }
+        }
+        if (cc < nch) {  // the plan's last group may hold fewer channels
+#pragma unroll
+            for (int i = 0; i < DPT; ++i) {
+                float v[SPT];
+                const T *t = s + offs[cc * Dt + i];
+#pragma unroll
+                for (int j = 0; j < SPT; ++j) v[j] = __fmul_rn(sw[cc], Elem<T>::val(t[32 * j]));
+#pragma unroll 1
+                for (int c = cc + 1; c < nch; ++c) {
+                    t = s + offs[c * Dt + i];
+#pragma unroll
+                    for (int j = 0; j < SPT; ++j)
+                        v[j] = __fmaf_rn(sw[c], Elem<T>::val(t[32 * j]), v[j]);
+                }
+#pragma unroll
+                for (int j = 0; j < SPT; ++j) acc[i][j] = __fadd_rn(acc[i][j], v[j]);
+            }
+        }
+    }
+};
+
 // kind 1: thread-contiguous samples served from a register window.
 template <typename T, int DPT, int SPT>
 struct RegWindow {
@@ -703,6 +767,7 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs &a, int dtile, int ttile,
     using Acc = typename Elem<T>::Acc;
     using Wt = typename Elem<T>::W;
     constexpr bool WIN = is_window(KIND, SPT), QUAD = is_quad(KIND, SPT);
+    constexpr bool GROUPS = sums_groups(KIND, DPT, SPT) && std::is_same<Acc, float>::value;
     // With two slots, a refill at the end of a chunk leaves no copy in flight
     // during the next one; the kernels with the largest tiles, whose slots
     // leave no room for a third, refill before they sum a chunk (LOFAR, 8
@@ -809,6 +874,8 @@ __device__ __forceinline__ void fwd_tile(const FwdArgs &a, int dtile, int ttile,
                 Quads<SPT>::template chunk<true>(acc, sdata + lb, soffs, a.Dt, sw, nch);
             else
                 Quads<SPT>::template chunk<false>(acc, sdata + lb, soffs, a.Dt, sw, nch);
+        } else if constexpr (GROUPS) {
+            GroupedLanes<T, DPT, SPT>::chunk(acc, sdata + lb, soffs, a.Dt, sw, nch);
         } else {
             for (int cc = 0; cc < nch; ++cc) {
                 int o[DPT];

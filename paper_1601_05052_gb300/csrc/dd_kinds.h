@@ -33,6 +33,13 @@ __host__ __device__ constexpr bool is_window(int kind, int spt) {
 // Byte-quad form of kind 0 (8-bit input only): 20 consecutive samples per
 // thread, read as 32-bit words.
 __host__ __device__ constexpr bool is_quad(int kind, int spt) { return kind == 0 && spt == 20; }
+// Forms of float input that sum groups of four consecutive channels before they
+// add to the accumulators, in the sub-bands' order: the sub-bands themselves and
+// the lane-strided 2 x 4, 4 x 2 and 4 x 8. Their rounding error over C channels
+// grows like that of a chain of C / 4 terms, the other forms' like C terms.
+__host__ __device__ constexpr bool sums_groups(int kind, int dpt, int spt) {
+    return is_subband(kind) || (kind == 0 && (dpt * spt == 8 || (dpt == 4 && spt == 8)));
+}
 // Kernels whose CTAs may have 16 trial warps and stage 1 or 2 channels at a time:
 // the register windows, the byte quads and the lane-strided 8 x 8 form.
 __host__ __device__ constexpr bool is_wide(int kind, int dpt, int spt) {
@@ -49,11 +56,14 @@ __host__ __device__ constexpr int max_trial_warps(int kind, int dpt, int spt) {
     return (kind == 4 || kind == 6 || is_wide(kind, dpt, spt)) ? 16 : 8;
 }
 // Launch bounds of the forward kernels: threads per CTA and resident CTAs
-// per SM that the register allocation must allow.
+// per SM that the register allocation must allow (the lane-strided 4 x 8 form's
+// grouped sums would take 140 registers instead of 128, one CTA of four warps
+// fewer per SM).
 __host__ __device__ constexpr int fwd_max_threads(int kind, int dpt, int spt) {
     return 32 * (max_trial_warps(kind, dpt, spt) + extra_warps(kind));
 }
 __host__ __device__ constexpr int fwd_min_blocks(int kind, int dpt, int spt) {
+    if (kind == 0 && dpt == 4 && spt == 8) return 2;
     return kind == 2 ? (dpt * spt <= 16 ? 3 : 2) : (kind == 3 ? 2 : 1);
 }
 

@@ -1,0 +1,90 @@
+/* The CUDA runtime calls that libdd.so makes while it plans, answered on the
+ * host as a GB300 would answer them, for tests of plan-time decisions on a
+ * machine without a GPU (preloaded before the real runtime, which still
+ * registers the kernels). Nothing runs: "device" memory is host memory that no
+ * one reads, launches are only recorded. */
+#include <stdlib.h>
+#include <string.h>
+
+typedef int err_t;
+typedef struct { unsigned x, y, z; } dim3_t;
+/* one recorded launch: shape and the first bytes of the first argument */
+typedef struct {
+    dim3_t grid, block;
+    size_t smem;
+    unsigned char arg0[256];
+} launch_t;
+
+static launch_t launches[64];
+static int n_launches;
+
+int fake_launch_count(void) { return n_launches; }
+const launch_t *fake_launch(int i) { return &launches[i]; }
+void fake_launch_reset(void) { n_launches = 0; }
+
+err_t cudaGetDevice(int *d) { *d = 0; return 0; }
+err_t cudaDeviceGetAttribute(int *v, int attr, int d) {
+    *v = attr == 16 ? 152 : (attr == 97 ? 227 * 1024 : 0); /* SMs, shared memory per block */
+    return 0;
+}
+err_t cudaGetDeviceProperties(void *p, int d) {
+    memset(p, 0, 256); /* the name comes first */
+    strcpy(p, "fake");
+    return 0;
+}
+err_t cudaStreamCreateWithFlags(void **s, unsigned f) { *s = NULL; return 0; }
+err_t cudaStreamDestroy(void *s) { return 0; }
+err_t cudaStreamSynchronize(void *s) { return 0; }
+err_t cudaStreamWaitEvent(void *s, void *e, unsigned f) { return 0; }
+err_t cudaStreamIsCapturing(void *s, int *st) { *st = 0; return 0; }
+err_t cudaDeviceSynchronize(void) { return 0; }
+err_t cudaEventCreate(void **e) { *e = (void *)1; return 0; }
+err_t cudaEventCreateWithFlags(void **e, unsigned f) { *e = (void *)1; return 0; }
+err_t cudaEventDestroy(void *e) { return 0; }
+err_t cudaEventRecord(void *e, void *s) { return 0; }
+err_t cudaEventSynchronize(void *e) { return 0; }
+static err_t allocate(void **p) { return posix_memalign(p, 256, 256) ? 2 : 0; }
+err_t cudaMalloc(void **p, size_t n) { return allocate(p); }
+err_t cudaMallocAsync(void **p, size_t n, void *s) { return allocate(p); }
+err_t cudaFree(void *p) { free(p); return 0; }
+err_t cudaFreeAsync(void *p, void *s) { free(p); return 0; }
+err_t cudaMemcpy(void *a, const void *b, size_t n, int k) { return 0; }
+err_t cudaMemcpyAsync(void *a, const void *b, size_t n, int k, void *s) { return 0; }
+err_t cudaMemset(void *a, int v, size_t n) { return 0; }
+err_t cudaMemsetAsync(void *a, int v, size_t n, void *s) { return 0; }
+err_t cudaFuncGetAttributes(void *a, const void *f) { memset(a, 0, 64); return 0; }
+err_t cudaFuncSetAttribute(const void *f, int a, int v) { return 0; }
+err_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int *n, const void *f, int b, size_t s) {
+    *n = 1;
+    return 0;
+}
+err_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *f, int b, size_t s,
+                                                             unsigned fl) {
+    *n = 1;
+    return 0;
+}
+err_t cudaGraphCreate(void **g, unsigned f) { *g = (void *)1; return 0; }
+err_t cudaGraphAddMemsetNode(void **n, void *g, void *const *d, size_t k, const void *p) {
+    *n = (void *)1;
+    return 0;
+}
+err_t cudaGraphAddKernelNode(void **n, void *g, void *const *d, size_t k, const void *p) {
+    *n = (void *)1;
+    return 0;
+}
+err_t cudaGraphInstantiate(void **e, void *g, unsigned long long f) { *e = (void *)1; return 0; }
+err_t cudaGraphExecDestroy(void *e) { return 0; }
+err_t cudaGraphDestroy(void *g) { return 0; }
+err_t cudaGetLastError(void) { return 0; }
+err_t __cudaGetKernel(void **k, const void *f) { *k = (void *)f; return 0; }
+err_t __cudaLaunchKernel(void *f, dim3_t grid, dim3_t block, void **args, size_t smem, void *s) {
+    if (n_launches < 64) {
+        launch_t *l = &launches[n_launches++];
+        l->grid = grid;
+        l->block = block;
+        l->smem = smem;
+        memcpy(l->arg0, args[0], 8); /* every kernel's first argument has 8 bytes */
+        if (smem) memcpy(l->arg0, args[0], sizeof l->arg0); /* forward kernels: FwdArgs */
+    }
+    return 0;
+}

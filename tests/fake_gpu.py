@@ -1,0 +1,125 @@
+"""Plan-time decisions of libdd.so on a machine without a GPU: a child process
+preloads fake_cudart.c, makes plans and batches and reports what they start
+with. (Run as a program this file is that child.)"""
+import ctypes
+import json
+import os
+import subprocess
+import sys
+import types
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+PACKAGE = "paper_1601_05052_gb300"
+# band: lowest channel MHz, band top MHz, sampling time s, trial DM step
+BANDS = {"lband": (1400.0, 1500.0, 64e-6, 0.5), "apertif": (1420.0, 1720.0, 50e-6, 0.25),
+         "wide": (1250.0, 1550.0, 100e-6, 0.25), "lowfreq": (120.0, 180.0, 204.8e-6, 0.05),
+         "lofar": (138.0, 144.25, 5e-6, 0.25)}
+
+
+def probe(requests, tmp_path):
+    """Answers of the child to each request {"setups": [[band, beams, channels,
+    trials, samples, type], ...], "ask": [...]}."""
+    from paper_1601_05052_gb300 import _build
+    _build.build()
+    so = os.path.join(str(tmp_path), "libfake_cudart.so")
+    subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-w", "-o", so,
+                    os.path.join(HERE, "fake_cudart.c")], check=True)
+    env = dict(os.environ, LD_PRELOAD=so, FAKE_CUDART=so)
+    env.pop("DD_TUNE_CACHE", None)
+    r = subprocess.run([sys.executable, os.path.abspath(__file__)], input=json.dumps(requests),
+                       capture_output=True, text=True, env=env, timeout=300)
+    assert r.returncode == 0, r.stderr[-3000:]
+    return json.loads(r.stdout)
+
+
+class FwdArgsHead(ctypes.Structure):
+    """The leading members of a forward kernel's argument (dd_fwd_tile.cuh)."""
+    _fields_ = ([("in_", ctypes.c_void_p), ("w", ctypes.c_void_p), ("out", ctypes.c_void_p),
+                 ("C", ctypes.c_int32), ("D", ctypes.c_int32),
+                 ("S", ctypes.c_int64), ("stride", ctypes.c_int64)]
+                + [(n, ctypes.c_int32) for n in
+                   "Dt Ts C_pad cch stages warps_dm stage_data stage_offs n_dtiles n_ttiles B "
+                   "ttile0 dtile0 grid_tt grid_dt time_major".split()])
+
+
+class Launch(ctypes.Structure):
+    _fields_ = [("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3),
+                ("smem", ctypes.c_size_t), ("arg0", ctypes.c_ubyte * 256)]
+
+
+def _child():
+    # the package's binding without its __init__, which needs torch
+    pkg = types.ModuleType(PACKAGE)
+    pkg.__path__ = [os.path.join(ROOT, PACKAGE)]
+    sys.modules[PACKAGE] = pkg
+    sys.path.insert(0, ROOT)
+    import importlib
+    L = importlib.import_module(PACKAGE + "._lib")
+    lib = L.load()
+    fake = ctypes.CDLL(os.environ["FAKE_CUDART"])
+    fake.fake_launch.restype = ctypes.POINTER(Launch)
+
+    def plan(band, beams, chan, dm, out, dtype):
+        lo, hi, t_samp, step = BANDS[band]
+        f = (ctypes.c_double * chan)(*[lo + c * (hi - lo) / chan for c in range(chan)])
+        d = (ctypes.c_double * dm)(*[i * step for i in range(dm)])
+        p = ctypes.c_void_p()
+        L.check(lib.dd_plan_create(ctypes.byref(p), chan, f, hi - (hi - lo) / chan, t_samp, dm, d,
+                                   out, beams, L.DTYPES[dtype]))
+        return p
+
+    def variant(fn, *args):
+        v = L.Variant()
+        L.check(fn(*args, ctypes.byref(v)))
+        return list(v.as_tuple())
+
+    def order(p):
+        o = ctypes.c_int32()
+        L.check(lib.dd_plan_get_launch_order(p, ctypes.byref(o)))
+        return o.value
+
+    def launches(call):
+        fake.fake_launch_reset()
+        L.check(call())
+        res = []
+        for i in range(fake.fake_launch_count()):
+            x = fake.fake_launch(i).contents
+            e = {"grid": list(x.grid), "block": list(x.block), "smem": x.smem}
+            if x.smem:
+                a = FwdArgsHead.from_buffer_copy(bytes(x.arg0))
+                e["args"] = {n: getattr(a, n) for n, _ in FwdArgsHead._fields_[3:]}
+            res.append(e)
+        return res
+
+    answers = []
+    buf = ctypes.create_string_buffer(4096)
+    ptr = ctypes.c_void_p((ctypes.addressof(buf) + 255) & ~255)
+    for req in json.loads(sys.stdin.read()):
+        plans = [plan(*s) for s in req["setups"]]
+        ans = {"plans": [variant(lib.dd_plan_get_variant, p) for p in plans],
+               "orders": [order(p) for p in plans]}
+        ask = req.get("ask", [])
+        if "adjoint" in ask:
+            ans["adjoint"] = variant(lib.dd_adjoint_get_variant, plans[0])
+            ans["adjoint_launches"] = launches(
+                lambda: lib.dd_adjoint(plans[0], ptr, ptr, ptr, ptr, None, None))
+        if "batch" in ask:
+            b = ctypes.c_void_p()
+            L.check(lib.dd_batch_create(ctypes.byref(b), len(plans),
+                                        (ctypes.c_void_p * len(plans))(*[p.value for p in plans])))
+            ans["batch"] = variant(lib.dd_batch_get_variant, b)
+            lib.dd_batch_destroy(b)
+        if "stream" in ask:
+            s = ctypes.c_void_p()
+            L.check(lib.dd_stream_create(ctypes.byref(s), plans[0]))
+            ans["stream_launches"] = launches(lambda: lib.dd_stream_push(s, ptr, ptr, ptr, None))
+            lib.dd_stream_destroy(s)
+        for p in plans:
+            lib.dd_plan_destroy(p)
+        answers.append(ans)
+    print(json.dumps(answers))
+
+
+if __name__ == "__main__":
+    _child()

@@ -1,0 +1,50 @@
+"""What plans start with, decided without a GPU (fake_gpu.py): float sums keep
+the grouping that the sub-band kernels give them."""
+import pytest
+
+from fake_gpu import probe
+
+SUBBANDS = (2, 3, 4, 6)
+
+
+def grouped(v):
+    """Whether a variant sums groups of four channels before it accumulates."""
+    kind, dpt, spt = v[:3]
+    return kind in SUBBANDS or (kind == 0 and (dpt * spt == 8 or (dpt, spt) == (4, 8)))
+
+
+# Setups whose channel groups share few delay patterns, so that a sub-band
+# variant fits them: few and many trials, few and many channels.
+GROUPED = [
+    ("apertif", 1, 1024, 16, 20000, "f32"), ("apertif", 2, 1024, 8, 20000, "f16"),
+    ("wide", 4, 512, 20, 8192, "f32"), ("wide", 16, 300, 4, 8192, "bf16"),
+    ("lband", 384, 64, 4, 4096, "f32"), ("lband", 303, 40, 7, 1934, "f32"),
+    ("lband", 72, 88, 7, 5162, "bf16"), ("lband", 7, 80, 37, 8030, "f32"),
+    ("lband", 99, 92, 27, 5988, "f32"), ("lband", 238, 72, 22, 3260, "f32"),
+    ("lband", 247, 120, 67, 1347, "f32"), ("wide", 8, 219, 101, 9289, "f32"),
+    ("apertif", 1, 1024, 2048, 20000, "f32"), ("wide", 2, 509, 777, 10001, "f16"),
+]
+# No sub-band variant fits these; one chain over the channels is all they ever had.
+FREE = [("lband", 96, 64, 64, 4096, "f32"), ("lofar", 1, 32, 2048, 200000, "f32")]
+
+
+@pytest.fixture(scope="module")
+def answers(tmp_path_factory):
+    req = [{"setups": [s], "ask": ["adjoint"] if s[5] == "f32" else []} for s in GROUPED + FREE]
+    return dict(zip(GROUPED + FREE, probe(req, tmp_path_factory.mktemp("fake"))))
+
+
+@pytest.mark.parametrize("setup", GROUPED, ids=str)
+def test_float_sums_keep_their_channel_groups(answers, setup):
+    assert grouped(answers[setup]["plans"][0]), answers[setup]
+
+
+@pytest.mark.parametrize("setup", [s for s in GROUPED if s[5] == "f32" and s[2] > 128], ids=str)
+def test_adjoint_sums_keep_their_groups(answers, setup):
+    """The transposed plan sums over trials; at these bands its groups of four
+    trials share few patterns too."""
+    assert grouped(answers[setup]["adjoint"]), answers[setup]
+
+
+def test_plans_without_sub_bands_may_chain(answers):
+    assert [answers[s]["plans"][0][:3] for s in FREE] == [[5, 4, 22], [0, 8, 8]]
