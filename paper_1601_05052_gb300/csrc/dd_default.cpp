@@ -2,21 +2,25 @@
 // of the candidate variants, from the plan's sizes, type and delay steps.
 //
 // One tile of a variant takes, with r CTAs resident on its SM,
-//     max(r * warps * C * (a (W + G) + b + 10 k / cch), C (10 l + 100 m / cch)) + 1000 o
+//     max(r * warps * C * (a (W + G) + s P + b + 10 k / cch), C (10 l + 100 m / cch)) + 1000 o
 // clocks: its share of the SM's shared-memory pipe and issue slots, or the
 // latency of one channel after the other when too few warps are resident,
 // plus a tile's start and end. W is the shared-memory words a warp reads per
-// channel, G the staged words, cch the channels per stage. The tiles run in
-// rounds of the CTAs that are resident at once; staged bytes (L2) and
-// compulsory bytes (HBM) bound the sum from below. The constants of each
-// kernel family were fitted on a GB300 to timings of 272 setups drawn from
-// five bands (64-channel L-band, Apertif, 300 MHz L-band, 120-180 MHz, LOFAR;
-// 1 to 384 beams, 16 to 1024 channels, 4 to 2048 trials, all four input types),
-// each with every candidate that fits it. Residual 6 % (quads) and 10 %
-// (lane-strided, windows) to 15 % (sub-bands, whose patterns are not counted). Over
-// those setups the model's choice took 1.03 times the best candidate's time in
-// the geometric mean (1.31 at worst); the fixed preference list it replaced,
-// 1.39 times (5.2 at worst, LOFAR).
+// channel, G the staged words, P the sub-bands' partial-series words, cch the
+// channels per stage. The tiles run in rounds of the CTAs that are resident at
+// once; staged bytes (L2) and compulsory bytes (HBM) bound the sum from below.
+// (Lane-strided with two small slots: latency s more, as no copy is in flight
+// while a chunk is summed.)
+// The constants of each kernel family were fitted on a GB300 to 66900 timings
+// (44 variants, where they fit, on 2439 setups: 2036 drawn from five bands, 1 to
+// 384 beams, 16 to 1024 channels, 4 to 2048 trials, all input types, the
+// gradients' transposed tables too; 403 at steps of up to 1.5 samples), then
+// adjusted, on four fifths of the setups, to what the choice costs. Residuals
+// 11 % (windows) to 20 % (kind 4). The choice, among the variants that keep a
+// plan's channel groups (dd_plan.cpp), takes 1.017 times the best one's time in
+// the geometric mean (1.017 on the last fifth too), 1.12 at the 95th percentile
+// and 1.63 at worst. (1.041 and 2.67 with register counts that ptxas
+// contradicts, corrected by rules on channels, trials and steps.)
 #include <algorithm>
 #include <cmath>
 
@@ -31,8 +35,8 @@ struct Candidate {
     bool time_major;
 };
 
-// The variants worth starting with: of 45 timed, these were within 0.3 % of
-// the best in the geometric mean.
+// The variants worth starting with: the best of them takes 1.005 times the best
+// of all 44 in the geometric mean.
 const Candidate kCandidates[] = {
     // sub-bands: long Eq. 1 grids whose channel groups share delay patterns
     {{6, 4, 8, 16, 1, 32, 2}, false},
@@ -67,6 +71,7 @@ const Candidate kCandidates[] = {
     {{0, 4, 8, 1, 8, 4, 3}, false},
     {{0, 4, 8, 4, 1, 8, 3}, false},
     {{0, 4, 8, 2, 4, 8, 3}, false},
+    {{0, 4, 8, 2, 2, 8, 3}, false},
     {{0, 4, 4, 4, 1, 16, 4}, false},
     {{0, 4, 2, 4, 2, 32, 2}, false},
     {{0, 2, 4, 4, 1, 32, 3}, false},
@@ -74,27 +79,30 @@ const Candidate kCandidates[] = {
     {{5, 4, 8, 4, 1, 16, 3}, false},
 };
 
-// Fitted constants {a, b, k, l, o, s, m}; s: sub-band build words.
+// Fitted constants of a kernel family.
 struct Fit {
     double a, b, k, l, o, s, m;
 };
-constexpr Fit kLane{0.95, 3.82, 1.55, 4.97, 6.49, 0, 13.84};
-constexpr Fit kQuad{1.3, 15.7, 2.84, 41.3, 6.12, 0, 7.05};
-constexpr Fit kWindow{1.21, 8.26, 0, 32.3, 9.1, 0, 8.41};
-constexpr Fit kReuse{0.58, 11.6, 11.2, 22.9, 3.93, 0, 34.8};
-constexpr Fit kSub2{1.03, 4.96, 0.73, 34.8, 1.84, 10.8, 3.44};
-constexpr Fit kSub4{0.28, 10.9, 2.17, 19.5, 2.02, 27.6, 15.7};
-constexpr Fit kSub6{0.06, 9.76, 8.19, 24.1, 2.69, 148, 3.01};
+constexpr Fit kLane{1.02, 0.47, 1.3, 3.01, 7.05, 128.67, 13.03};
+constexpr Fit kQuad{0.92, 20.68, 3.34, 23.41, 11.85, 0, 10.12};
+constexpr Fit kWindow{1.08, 1.32, 10.44, 39.46, 8.79, 0, 10.97};
+constexpr Fit kReuse{0.6, 5.15, 20, 13.09, 8.18, 0, 35.74};
+constexpr Fit kSub2{1.81, 0.17, 12.18, 17.93, 6.43, 2.09, 19.16};
+constexpr Fit kSub4{0.82, 5.23, 3.48, 18.56, 8.44, 6.35, 6.62};
+constexpr Fit kSub6{1.28, 0.83, 0.72, 5.08, 9.39, 7.49, 0.51};
 
-// Registers per thread of the kernels with 2x4 .. 8x8 outputs per thread.
-int registers(const dd_variant &v) {
-    if (v.kind == 2) return v.dm_per_thread * v.samples_per_thread <= 16 ? 72 : 80;
+// Registers per thread of the candidates' one-shot kernels, as ptxas reports
+// them (asking the runtime would load every candidate's code at plan time).
+int registers(dd_dtype t, const dd_variant &v) {
+    const int n = v.dm_per_thread * v.samples_per_thread;
+    if (v.kind == 2) return n <= 16 ? 72 : 96;
     if (v.kind == 4 || v.kind == 6) return 96;
     if (is_window(v.kind, v.samples_per_thread) || is_quad(v.kind, v.samples_per_thread))
         return 128;
-    if (v.kind == 5) return 90;
-    const int n = v.dm_per_thread * v.samples_per_thread;
-    return n <= 8 ? 40 : (n <= 16 ? 56 : (n <= 32 ? 76 : 126));
+    if (v.kind == 5) return 88;
+    if (n <= 8) return t == DD_F32 ? 118 : 96;
+    if (n <= 16) return 96;
+    return n <= 32 && t == DD_U8 ? 106 : 128;
 }
 
 }  // namespace
@@ -139,18 +147,18 @@ double model_us(const dd_plan_s *p, const DelaySteps &st, const dd_variant &v) {
     const double slot = std::min(cch, C) * widest * elt + cch * (2 * Dt + 20);
     double smem = 1152 + v.stages * slot;
     if (sb) {  // partial series, at five patterns per group
-        const double P = cch / 4 * 5 * (Ts + De * st.max) * 4 * 1.15;
-        smem += v.kind == 6 ? P : 2 * P;
+        const double series = cch / 4 * 5 * (Ts + De * st.max) * 4 * 1.15;
+        smem += v.kind == 6 ? series : 2 * series;
     }
     const int threads = 32 * (nw + extra_warps(v.kind));
     const double r_max = std::max(
-        1.0, std::floor(std::min({233000.0 / smem,
-                                  65536.0 / ((registers(v) + 7) / 8 * 8 * threads),
+        1.0, std::floor(std::min({double(p->smem_optin + 1024) / smem,
+                                  65536.0 / ((registers(p->dtype, v) + 7) / 8 * 8 * threads),
                                   2048.0 / threads, 32.0})));
     // Words per warp and channel. Shared operands: steps taken as spread
     // evenly over [0, 2 mean], `same` of adjacent trials share a delay.
     const double x = 2 * st.mean, same = x <= 1 ? 1 - x / 2 : 1 / (2 * x);
-    double W = v.dm_per_thread * v.samples_per_thread;
+    double W = v.dm_per_thread * v.samples_per_thread, P = 0;
     if (quad)
         W = v.dm_per_thread * (v.samples_per_thread / 4 + 1);
     else if (win && st.max <= kWinBands + 0.5)
@@ -158,9 +166,11 @@ double model_us(const dd_plan_s *p, const DelaySteps &st, const dd_variant &v) {
     else if (v.kind == 5 && !win)
         W *= 1 - same * (v.dm_per_thread - 1) / v.dm_per_thread;
     else if (sb)
-        W = W / 4 * (1 - same / 2) + f.s * (Ts + De * st.mean) / (32 * nw);
-    const double per = C * (f.a * (W + len * elt / 128 / nw) + f.b + 10 * f.k / cch);
-    const double lat = C * (10 * f.l + 100 * f.m / cch);
+        W = W / 4 * (1 - same / 2), P = (Ts + De * st.mean) / (32 * nw);
+    const double per = C * (f.a * (W + len * elt / 128 / nw) + f.s * P + f.b + 10 * f.k / cch);
+    // two small slots leave no copy in flight while a chunk is summed
+    const bool bare = v.kind == 0 && v.stages == 2 && v.dm_per_thread * v.samples_per_thread < 64;
+    const double lat = C * (10 * f.l + 100 * f.m / cch + (bare ? f.s : 0));
     auto tile = [&](double r) { return std::max(r * nw * per, lat) + 1000 * f.o; };
     const double slots = r_max * p->sm_count, full = std::floor(tiles / slots);
     const double rest = tiles - full * slots;
@@ -170,17 +180,6 @@ double model_us(const dd_plan_s *p, const DelaySteps &st, const dd_variant &v) {
     us = std::max(us, tiles * C * len * elt / 7.5e6);
     us = std::max(us, (p->B * C * double(p->stride) * elt + 4.0 * p->B * p->D * double(p->S)) / 5.5e6);
     return us;
-}
-
-// Long float chains whose delays move by 12 to 32 samples per trial (adjoints
-// at survey bands; low bands start at 39): sub-bands round less there too, but
-// the model does not order them well enough (gradients of 3 x 268 channels x
-// 1886 trials x 10382 samples: its choice 5.8 ms, the preference list's 4.5;
-// windows 3.6 at twice the error).
-bool by_preference(const dd_plan_s *p) {
-    if (p->dtype == DD_U8 || p->C <= 128 || p->D < 24) return false;
-    const double steps = delay_steps(p).max;
-    return steps > 12 && steps <= 32;
 }
 
 std::vector<RankedVariant> ranked_variants(const dd_plan_s *p) {
@@ -194,25 +193,17 @@ std::vector<RankedVariant> ranked_variants(const dd_plan_s *p) {
         // One partial-sum slot only where two do not fit (survey scale, 8-bit:
         // kind 4 2.26 ms, kind 6 2.38; FP32 fits 32 channels in kind 6 alone).
         if (c.v.kind == 6 && c.v.warps_dm == 16 && p->dtype != DD_F32) continue;
-        // Where no channel moves by more than 0.8 samples per trial, a
-        // thread's trials mostly share a sub-band's series and offset, which
-        // the model does not see (500 channels x 1000 trials x 10000 samples,
-        // FP32: sub-bands 0.51 ms, windows 0.59, lane-strided 1.2). And a
-        // float chain over more than 128 channels rounds more than the
-        // sub-bands' groups of four, so smooth delays keep those: 473 channels
-        // x 788 trials x 4406 samples, gradients, 5.2e-7 of the largest output
-        // against 2.8e-7, and 0.69 ms against 0.55.
-        if (p->D >= 24 && !is_subband(c.v.kind) &&
-            (st.max <= 0.8 || (p->dtype != DD_U8 && p->C > 128 && st.max <= 12)))
-            continue;
-        // Near ties go to the wide sub-bands, whose grouped sums are also the
-        // more accurate (500 channels x 1000 trials, FP32: 0.54 ms where the
-        // model has 0.61, windows 0.615 where it has 0.56).
-        const double tie = is_subband(c.v.kind) && c.v.warps_dm == 16 ? 1.0 : 1.04;
-        r.push_back(RankedVariant{c.v, c.time_major, tie * model_us(p, st, c.v)});
+        r.push_back(RankedVariant{c.v, c.time_major, model_us(p, st, c.v)});
     }
-    std::stable_sort(r.begin(), r.end(),
-                     [](const RankedVariant &a, const RankedVariant &b) { return a.us < b.us; });
+    // 8-bit sums at nearly constant delays: sub-bands first, whose few series
+    // per group the model does not count (204 setups of 32 to 1024 channels and
+    // up to 1.5 samples per trial: choice 1.067 times the best, 1.05 with lines
+    // from 0.2 to 0.5, 1.061 at 0.8; floats do better without: 1.027 to 1.036).
+    const bool smooth = p->dtype == DD_U8 && p->D >= 24 && st.max <= 0.3;
+    std::stable_sort(r.begin(), r.end(), [&](const RankedVariant &a, const RankedVariant &b) {
+        if (smooth && is_subband(a.v.kind) != is_subband(b.v.kind)) return is_subband(a.v.kind);
+        return a.us < b.us;
+    });
     return r;
 }
 

@@ -222,7 +222,6 @@ struct RankedVariant {
 };
 // The candidate variants, fastest by the model first (they may not fit).
 std::vector<RankedVariant> ranked_variants(const dd_plan_s *p);
-bool by_preference(const dd_plan_s *p);  // the fixed preference list instead
 
 bool aligned16(const void *p);
 

@@ -543,30 +543,29 @@ dd_status build_default(dd_plan_s *p, FwdTables *out) {
     FwdTables sub;                          // the list's first sub-band variant that fits
     bool looked = p->dtype == DD_U8, grouped = false;  // whole numbers: any order
     dd_status s = DD_ERR_ARG;
-    if (!by_preference(p))
-        for (const RankedVariant &r : ranked_variants(p)) {
-            const dd_variant &v = r.v;
-            if (!sums_groups(v.kind, v.dm_per_thread, v.samples_per_thread) && !looked) {
-                looked = true;
-                for (const dd_variant &d : kDefaults) {
-                    if (!is_subband(d.kind)) break;
-                    s = build_fwd_tables(p, d, &sub);
-                    if (s != DD_OK && s != DD_ERR_ARG) return s;
-                    grouped = s == DD_OK;
-                    if (grouped) break;
-                }
+    for (const RankedVariant &r : ranked_variants(p)) {
+        const dd_variant &v = r.v;
+        if (!sums_groups(v.kind, v.dm_per_thread, v.samples_per_thread) && !looked) {
+            looked = true;
+            for (const dd_variant &d : kDefaults) {
+                if (!is_subband(d.kind)) break;
+                s = build_fwd_tables(p, d, &sub);
+                if (s != DD_OK && s != DD_ERR_ARG) return s;
+                grouped = s == DD_OK;
+                if (grouped) break;
             }
-            if (grouped && !sums_groups(v.kind, v.dm_per_thread, v.samples_per_thread)) continue;
-            if (grouped && std::memcmp(&v, &sub.v, sizeof v) == 0) {
-                *out = sub;
-                return DD_OK;
-            }
-            s = build_fwd_tables(p, v, out);
-            if (s == DD_ERR_ARG) continue;
-            if (grouped) free_fwd_tables(&sub);
-            out->time_major = s == DD_OK && r.time_major;
-            return s;
         }
+        if (grouped && !sums_groups(v.kind, v.dm_per_thread, v.samples_per_thread)) continue;
+        if (grouped && std::memcmp(&v, &sub.v, sizeof v) == 0) {
+            *out = sub;
+            return DD_OK;
+        }
+        s = build_fwd_tables(p, v, out);
+        if (s == DD_ERR_ARG) continue;
+        if (grouped) free_fwd_tables(&sub);
+        out->time_major = s == DD_OK && r.time_major;
+        return s;
+    }
     if (grouped) {
         *out = sub;
         return DD_OK;

@@ -1,5 +1,6 @@
 """What plans start with, decided without a GPU (fake_gpu.py): float sums keep
-the grouping that the sub-band kernels give them."""
+the grouping that the sub-band kernels give them, and the time model orders
+setups whose fastest variants are known from timings."""
 import pytest
 
 from fake_gpu import probe
@@ -48,3 +49,24 @@ def test_adjoint_sums_keep_their_groups(answers, setup):
 
 def test_plans_without_sub_bands_may_chain(answers):
     assert [answers[s]["plans"][0][:3] for s in FREE] == [[5, 4, 22], [0, 8, 8]]
+
+
+# (setup, starting keys that timings on a GB300 bear out, launch order)
+SMALL = [[0, 2, 4], [0, 4, 2]]
+KNOWN = [
+    (("apertif", 1, 1024, 2048, 20000, "f32"), [[6, 4, 8]], 0),
+    (("apertif", 1, 1024, 2048, 20000, "u8"), [[4, 4, 8]], 0),
+    (("lband", 96, 64, 64, 4096, "f32"), [[5, 4, 22]], 0),
+    (("lband", 96, 64, 64, 4096, "u8"), [[0, 4, 20]], 0),
+    (("lofar", 1, 32, 2048, 200000, "f32"), [[0, 8, 8]], 1),
+    # one beam, few trials: small tiles (18 to 27 us) against sub-bands (44)
+    (("wide", 1, 281, 128, 2189, "f32"), SMALL, 0),
+    (("wide", 1, 150, 67, 2091, "f32"), SMALL, 0),
+    (("wide", 1, 223, 86, 2534, "bf16"), SMALL, 0),
+]
+
+
+def test_known_fastest_variants(tmp_path):
+    got = probe([{"setups": [s]} for s, _, _ in KNOWN], tmp_path)
+    for a, (setup, keys, order) in zip(got, KNOWN):
+        assert a["plans"][0][:3] in keys and a["orders"][0] == order, (setup, a)
