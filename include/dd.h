@@ -283,7 +283,8 @@ dd_status dd_adjoint_set_variant(dd_plan plan, const dd_variant *v);
  * warps (warps_dm * warps_time); each plan has its own split of those warps
  * (its DM x time tile) and its own chans_per_stage. A batch starts with the
  * first plan's variant if that was set or tuned and fits every plan, else with
- * the variant whose modelled time over all plans is smallest. */
+ * the variant whose modelled time over all plans is smallest (float sums keep
+ * the channel groups that a plan's own default would keep). */
 dd_status dd_batch_create(dd_batch *out, int32_t n, const dd_plan *plans);
 dd_status dd_batch_execute(dd_batch batch, const void *const *d_in,
                            const void *const *d_w, void *const *d_out, void *stream);

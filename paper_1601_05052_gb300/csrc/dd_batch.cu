@@ -239,11 +239,33 @@ std::vector<RankedVariant> common_variants(const std::vector<dd_plan> &plans) {
                 common.push_back(RankedVariant{r.v, false, 0.0});
     for (dd_plan p : plans) {
         const DelaySteps st = delay_steps(p);
-        for (RankedVariant &r : common) r.us += model_us(p, st, r.v);
+        for (RankedVariant &r : common) r.us += batch_factor(p->dtype, r.v) * model_us(p, st, r.v);
     }
     std::stable_sort(common.begin(), common.end(),
                      [](const RankedVariant &a, const RankedVariant &b) { return a.us < b.us; });
     return common;
+}
+
+// Sets the batch to the first common variant that fits (see dd_batch_create);
+// DD_ERR_ARG if none of the candidates does.
+dd_status configure_default(dd_batch_s *bt) {
+    const std::vector<RankedVariant> common = common_variants(bt->plans);
+    bool keep = false, looked = false;
+    dd_status s = DD_ERR_ARG;
+    for (int chains = 0; chains < 2; ++chains)  // 1: those passed over before
+        for (size_t i = 0; i < common.size() && s != DD_OK; ++i) {
+            const dd_variant &v = common[i].v;
+            const bool chain = !sums_groups(v.kind, v.dm_per_thread, v.samples_per_thread);
+            if (chain && !looked) {
+                looked = true;
+                for (size_t j = 0; j < bt->plans.size() && !keep; ++j) {
+                    const dd_status q = keeps_groups(bt->plans[j], &keep);
+                    if (q != DD_OK) return q;
+                }
+            }
+            if (chains == 0 ? !(chain && keep) : chain && keep) s = configure(bt, v);
+        }
+    return s;
 }
 
 // Work-list position of the caller's plan index u, or -1.
@@ -294,10 +316,11 @@ dd_status dd_batch_create(dd_batch *out, int32_t n, const dd_plan *plans) {
     }
     // The first plan's variant if it was set or tuned and fits every plan; else
     // the common variant with the smallest modelled time over all plans, among
-    // those that fit every plan; else any compiled variant that does.
+    // those that fit every plan and keep the channel groups of each float plan
+    // that has them on its own (dd_plan.cpp); else one that does not keep them;
+    // else any compiled variant that fits.
     dd_status s = plans[0]->chosen ? configure(bt, plans[0]->fwd.v) : DD_ERR_ARG;
-    const std::vector<RankedVariant> common = common_variants(bt->plans);
-    for (size_t i = 0; i < common.size() && s != DD_OK; ++i) s = configure(bt, common[i].v);
+    if (s != DD_OK) s = configure_default(bt);
     if (s != DD_OK) {
         const int nv = dd_variant_count();
         for (int i = 0; i < nv && s != DD_OK; ++i) {

@@ -182,6 +182,24 @@ double model_us(const dd_plan_s *p, const DelaySteps &st, const dd_variant &v) {
     return us;
 }
 
+// How much longer the persistent form of a variant's kernel runs than its
+// one-shot form's model says (other registers, spills; one launch for all
+// plans): the geometric means over 587 batches of two setups, every candidate
+// that fits both. With them the choice takes 1.03 times the best candidate's
+// time, without 1.10.
+double batch_factor(dd_dtype t, const dd_variant &v) {
+    const int n = v.dm_per_thread * v.samples_per_thread, i = t == DD_F32 ? 0 : (t == DD_U8 ? 2 : 1);
+    using Row = const double[3];  // FP32, 16-bit, 8-bit
+    static Row sub{1.05, 1.3, 1.37}, reuse{1.04, 1.22, 0.96}, lane8{1, 1.06, 1},
+        lane16{1.12, 1.22, 1.02}, lane32{0.9, 1.05, 0.97}, lane64{1.1, 1.36, 1.16};
+    if (is_subband(v.kind)) return sub[i];
+    if (is_quad(v.kind, v.samples_per_thread)) return 1.17;
+    if (is_window(v.kind, v.samples_per_thread))  // FP32 only
+        return v.samples_per_thread == 14 ? 1.14 : (v.samples_per_thread == 18 ? 1.5 : 1.8);
+    if (v.kind == 5) return reuse[i];
+    return n <= 8 ? lane8[i] : (n <= 16 ? lane16[i] : (n <= 32 ? lane32[i] : lane64[i]));
+}
+
 std::vector<RankedVariant> ranked_variants(const dd_plan_s *p) {
     const DelaySteps st = delay_steps(p);
     std::vector<RankedVariant> r;

@@ -1,6 +1,7 @@
 // dd_internal.h -- plan state and kernel-launch interfaces shared by the
 // translation units of libdd.so. Not part of the public ABI (see dd.h).
 #pragma once
+#include <atomic>
 #include <cuda_runtime.h>
 
 #include <cstddef>
@@ -150,6 +151,9 @@ struct dd_plan_s {
 
     dd::FwdTables fwd;
     bool chosen = false;  // fwd's variant was set, tuned or restored, not modelled
+    // whether a sub-band variant of the preference list fits (float plans; -1:
+    // nobody asked yet)
+    std::atomic<int> groups{-1};
     dd::AdjState adj;
     int32_t *d_shifts = nullptr;  // device copy of `shifts`
     int *d_err = nullptr;         // device error word (dd::kErr* bits)
@@ -215,6 +219,7 @@ struct DelaySteps {
 };
 DelaySteps delay_steps(const dd_plan_s *p);
 double model_us(const dd_plan_s *p, const DelaySteps &st, const dd_variant &v);
+double batch_factor(dd_dtype t, const dd_variant &v);  // persistent against one-shot form
 struct RankedVariant {
     dd_variant v;
     bool time_major;
@@ -222,6 +227,8 @@ struct RankedVariant {
 };
 // The candidate variants, fastest by the model first (they may not fit).
 std::vector<RankedVariant> ranked_variants(const dd_plan_s *p);
+// Whether defaults of this plan must sum groups of four channels (dd_plan.cpp).
+dd_status keeps_groups(dd_plan_s *p, bool *keeps);
 
 bool aligned16(const void *p);
 

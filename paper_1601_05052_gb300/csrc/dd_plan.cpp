@@ -533,6 +533,20 @@ void cache_store(const std::string &key, const dd_variant &v, bool time_major) {
 
 namespace {
 
+// Builds the preference list's first sub-band variant that fits a float plan;
+// DD_ERR_ARG if none does (or for 8-bit input, whose sums are exact in any
+// order). Remembers which in p->groups.
+dd_status build_list_subband(dd_plan_s *p, FwdTables *out) {
+    dd_status s = DD_ERR_ARG;
+    for (const dd_variant &d : kDefaults) {
+        if (p->dtype == DD_U8 || !is_subband(d.kind)) break;
+        s = build_fwd_tables(p, d, out);
+        if (s != DD_ERR_ARG) break;
+    }
+    if (s == DD_OK || s == DD_ERR_ARG) p->groups = s == DD_OK;
+    return s;
+}
+
 // The tables a plan starts with: the modelled candidates in their order, then
 // the preference list; DD_ERR_ARG if none fits. A float plan that a sub-band
 // variant of the list fits keeps sums in groups of four channels: candidates
@@ -540,33 +554,27 @@ namespace {
 // for the plans that have no such variant (384 beams x 64 channels x 4 trials:
 // largest error 8.2e-8 of the largest output in groups, 1.7e-7 in one chain).
 dd_status build_default(dd_plan_s *p, FwdTables *out) {
-    FwdTables sub;                          // the list's first sub-band variant that fits
-    bool looked = p->dtype == DD_U8, grouped = false;  // whole numbers: any order
+    FwdTables sub;  // the list's sub-band variant, once a chain stands next
     dd_status s = DD_ERR_ARG;
     for (const RankedVariant &r : ranked_variants(p)) {
         const dd_variant &v = r.v;
-        if (!sums_groups(v.kind, v.dm_per_thread, v.samples_per_thread) && !looked) {
-            looked = true;
-            for (const dd_variant &d : kDefaults) {
-                if (!is_subband(d.kind)) break;
-                s = build_fwd_tables(p, d, &sub);
-                if (s != DD_OK && s != DD_ERR_ARG) return s;
-                grouped = s == DD_OK;
-                if (grouped) break;
-            }
+        const bool chain = !sums_groups(v.kind, v.dm_per_thread, v.samples_per_thread);
+        if (chain && p->groups < 0) {
+            s = build_list_subband(p, &sub);
+            if (s != DD_OK && s != DD_ERR_ARG) return s;
         }
-        if (grouped && !sums_groups(v.kind, v.dm_per_thread, v.samples_per_thread)) continue;
-        if (grouped && std::memcmp(&v, &sub.v, sizeof v) == 0) {
+        if (chain && p->groups == 1) continue;
+        if (p->groups == 1 && std::memcmp(&v, &sub.v, sizeof v) == 0) {
             *out = sub;
             return DD_OK;
         }
         s = build_fwd_tables(p, v, out);
         if (s == DD_ERR_ARG) continue;
-        if (grouped) free_fwd_tables(&sub);
+        if (p->groups == 1) free_fwd_tables(&sub);
         out->time_major = s == DD_OK && r.time_major;
         return s;
     }
-    if (grouped) {
+    if (p->groups == 1) {
         *out = sub;
         return DD_OK;
     }
@@ -634,6 +642,18 @@ dd_status check_common(dd_plan *out, int32_t n_chan, int32_t n_dm, int64_t n_out
 }
 
 }  // namespace
+
+dd_status keeps_groups(dd_plan_s *p, bool *keeps) {
+    if (p->groups < 0) {
+        FwdTables t;
+        const dd_status s = build_list_subband(p, &t);
+        if (s == DD_OK) free_fwd_tables(&t);
+        if (s != DD_OK && s != DD_ERR_ARG) return s;
+    }
+    *keeps = p->groups == 1;
+    return DD_OK;
+}
+
 }  // namespace dd
 
 using namespace dd;

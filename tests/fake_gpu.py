@@ -19,7 +19,7 @@ BANDS = {"lband": (1400.0, 1500.0, 64e-6, 0.5), "apertif": (1420.0, 1720.0, 50e-
 
 def probe(requests, tmp_path):
     """Answers of the child to each request {"setups": [[band, beams, channels,
-    trials, samples, type], ...], "ask": [...]}."""
+    trials, samples, type], ...], "set": variant of the first plan, "ask": [...]}."""
     from paper_1601_05052_gb300 import _build
     _build.build()
     so = os.path.join(str(tmp_path), "libfake_cudart.so")
@@ -100,6 +100,8 @@ def _child():
         ans = {"plans": [variant(lib.dd_plan_get_variant, p) for p in plans],
                "orders": [order(p) for p in plans]}
         ask = req.get("ask", [])
+        if "set" in req:
+            L.check(lib.dd_plan_set_variant(plans[0], ctypes.byref(L.Variant(*req["set"]))))
         if "adjoint" in ask:
             ans["adjoint"] = variant(lib.dd_adjoint_get_variant, plans[0])
             ans["adjoint_launches"] = launches(

@@ -70,3 +70,35 @@ def test_known_fastest_variants(tmp_path):
     got = probe([{"setups": [s]} for s, _, _ in KNOWN], tmp_path)
     for a, (setup, keys, order) in zip(got, KNOWN):
         assert a["plans"][0][:3] in keys and a["orders"][0] == order, (setup, a)
+
+
+LBAND96 = ("lband", 96, 64, 64, 4096)
+WIDE4 = ("wide", 4, 512, 1000, 8192)
+LOWFREQ = ("lowfreq", 4, 208, 500, 4000)
+
+
+@pytest.fixture(scope="module")
+def batches(tmp_path_factory):
+    pairs = {"free + grouped": [LBAND96, WIDE4], "grouped + free": [WIDE4, LBAND96],
+             "grouped + free 2": [("lband", 43, 46, 17, 2000), LOWFREQ],
+             "free": [LBAND96, LOWFREQ]}
+    req = {(n, t): {"setups": [list(s) + [t] for s in p], "ask": ["batch"]}
+           for n, p in pairs.items() for t in ("f32", "f16", "u8")}
+    req["chosen"] = {"setups": [list(LBAND96) + ["f32"], list(WIDE4) + ["f32"]], "ask": ["batch"],
+                     "set": [5, 4, 14, 4, 1, 8, 3]}
+    return dict(zip(req, probe(list(req.values()), tmp_path_factory.mktemp("fake"))))
+
+
+@pytest.mark.parametrize("pair", ["free + grouped", "grouped + free", "grouped + free 2"])
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+def test_batches_keep_the_groups_of_every_plan(batches, pair, dtype):
+    """A float plan that keeps its channel groups alone keeps them in a batch,
+    whatever stands beside it."""
+    assert grouped(batches[pair, dtype]["batch"]), batches[pair, dtype]
+
+
+def test_batches_with_other_rules(batches):
+    """8-bit sums in any order, and the first plan's variant where the caller
+    set one."""
+    assert batches["free", "u8"]["batch"][:3] == [0, 4, 20]
+    assert batches["chosen"]["batch"] == [5, 4, 14, 4, 1, 8, 3]
