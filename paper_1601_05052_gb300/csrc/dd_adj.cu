@@ -149,8 +149,14 @@ dd_status ensure_adj_state(dd_plan_s *p) {
     a.plan->nz_lo = a.M;
     a.plan->nz_hi = a.M + p->S;
     {
-        const dd_variant v0 = a.plan->fwd.v;
-        s = dd_plan_set_variant(a.plan, &v0);
+        // the same variant in its launch order again: the tuner's or the
+        // default's, which dd_plan_set_variant would reset
+        FwdTables t;
+        s = build_fwd_tables(a.plan, a.plan->fwd.v, &t);
+        if (s == DD_OK) {
+            t.time_major = a.plan->fwd.time_major;
+            s = replace_fwd_tables(a.plan, &a.plan->fwd, t);
+        }
         if (s != DD_OK) {
             dd_plan_destroy(a.plan);
             return s;

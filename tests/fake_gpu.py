@@ -19,14 +19,15 @@ BANDS = {"lband": (1400.0, 1500.0, 64e-6, 0.5), "apertif": (1420.0, 1720.0, 50e-
 
 def probe(requests, tmp_path):
     """Answers of the child to each request {"setups": [[band, beams, channels,
-    trials, samples, type], ...], "set": variant of the first plan, "ask": [...]}."""
+    trials, samples, type], ...], "set": variant of the first plan, "transposed": variant and launch order that
+    a tuning cache holds for its adjoint's plan, "ask": [...]}."""
     from paper_1601_05052_gb300 import _build
     _build.build()
     so = os.path.join(str(tmp_path), "libfake_cudart.so")
     subprocess.run(["gcc", "-shared", "-fPIC", "-O1", "-w", "-o", so,
                     os.path.join(HERE, "fake_cudart.c")], check=True)
     env = dict(os.environ, LD_PRELOAD=so, FAKE_CUDART=so)
-    env.pop("DD_TUNE_CACHE", None)
+    env["DD_TUNE_CACHE"] = os.path.join(str(tmp_path), "tune_cache")
     r = subprocess.run([sys.executable, os.path.abspath(__file__)], input=json.dumps(requests),
                        capture_output=True, text=True, env=env, timeout=300)
     assert r.returncode == 0, r.stderr[-3000:]
@@ -92,6 +93,22 @@ def _child():
             res.append(e)
         return res
 
+    def cache_transposed(p, setup, entry):
+        """A tuning-cache line for the adjoint's plan: D channels, C trials,
+        delays M - delay over the padded input rows."""
+        _, beams, chan, dm, _, _ = setup
+        sh = (ctypes.c_int32 * (chan * dm))()
+        L.check(lib.dd_plan_shifts(p, sh))
+        m = (max(sh) + 3) // 4 * 4
+        h = 1469598103934665603
+        for c in range(chan):
+            for d in range(dm):
+                for byte in (m - sh[d * chan + c]).to_bytes(4, "little"):
+                    h = (h ^ byte) * 1099511628211 % (1 << 64)
+        key = "fake/t0/C%d/D%d/S%d/B%d/%x" % (dm, chan, lib.dd_plan_input_stride(p), beams, h)
+        with open(os.environ["DD_TUNE_CACHE"], "a") as f:
+            f.write(" ".join([key] + [str(x) for x in entry]) + "\n")
+
     answers = []
     buf = ctypes.create_string_buffer(4096)
     ptr = ctypes.c_void_p((ctypes.addressof(buf) + 255) & ~255)
@@ -102,6 +119,8 @@ def _child():
         ask = req.get("ask", [])
         if "set" in req:
             L.check(lib.dd_plan_set_variant(plans[0], ctypes.byref(L.Variant(*req["set"]))))
+        if "transposed" in req:
+            cache_transposed(plans[0], req["setups"][0], req["transposed"])
         if "adjoint" in ask:
             ans["adjoint"] = variant(lib.dd_adjoint_get_variant, plans[0])
             ans["adjoint_launches"] = launches(

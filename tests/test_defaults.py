@@ -102,3 +102,15 @@ def test_batches_with_other_rules(batches):
     set one."""
     assert batches["free", "u8"]["batch"][:3] == [0, 4, 20]
     assert batches["chosen"]["batch"] == [5, 4, 14, 4, 1, 8, 3]
+
+
+@pytest.mark.parametrize("order", [0, 1])
+def test_adjoint_keeps_its_launch_order(tmp_path, order):
+    """The adjoint's plan starts in the launch order that goes with its
+    variant (here a tuning cache's), and its launch uses that order."""
+    setup = ("lofar", 1, 8, 16, 3000, "f32")
+    v = [0, 4, 4, 2, 2, 4, 3]
+    got = probe([{"setups": [setup], "transposed": v + [order], "ask": ["adjoint"]}], tmp_path)[0]
+    args = [x["args"] for x in got["adjoint_launches"] if "args" in x]
+    assert len(args) == 1 and (args[0]["C"], args[0]["D"]) == (16, 8)
+    assert got["adjoint"] == v and args[0]["time_major"] == order, got
