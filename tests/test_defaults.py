@@ -114,3 +114,14 @@ def test_adjoint_keeps_its_launch_order(tmp_path, order):
     args = [x["args"] for x in got["adjoint_launches"] if "args" in x]
     assert len(args) == 1 and (args[0]["C"], args[0]["D"]) == (16, 8)
     assert got["adjoint"] == v and args[0]["time_major"] == order, got
+
+
+@pytest.mark.parametrize("setup,least", [(("lofar", 1, 32, 2048, 200000, "f32"), 1000),
+                                         (("lofar", 1, 16, 64, 1000, "u8"), 16),
+                                         (("wide", 1, 512, 1024, 4096, "bf16"), 512)], ids=str)
+def test_stream_fill_covers_the_machine(tmp_path, setup, least):
+    """A push with few long rows fills its buffer with several blocks per row
+    (152 SMs), one with many short rows with one per row."""
+    fill = probe([{"setups": [setup], "ask": ["stream"]}], tmp_path)[0]["stream_launches"][0]
+    assert fill["smem"] == 0 and fill["grid"][0] == setup[1] * setup[2]
+    assert least <= fill["grid"][0] * fill["grid"][1] <= max(least, 16 * 152), fill
