@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "dd_internal.h"
@@ -193,21 +194,25 @@ extern "C" dd_status dd_tune(dd_plan p, int32_t budget_ms, dd_tune_report *rep) 
         *ms = total / reps;
         return DD_OK;
     };
-    // Launch order of the timed launches: DM tiles fastest in pass 1; pass
-    // 1's winner is then timed in both orders and pass 2 (the staging
-    // choices) runs in the faster one, since the order decides what stays in
-    // L2 and so which staging depth pays.
-    bool order_time = false;
+    // Launch order of the timed launches: DM tiles fastest in pass 1 (a modelled
+    // candidate's own order for that candidate); pass 1's winner is then timed in
+    // both orders and pass 2 (the staging choices) runs in the faster one, since
+    // the order decides what stays in L2 and so which staging depth pays.
+    const std::vector<RankedVariant> ranked = ranked_variants(p);
+    bool order_time = false, settled = false;
     auto time_ms = [&](const dd_variant &v, double *ms) -> dd_status {
         FwdTables t;
         if (build_fwd_tables(p, v, &t) != DD_OK) return DD_OK;  // does not fit: not meaningful
         t.time_major = order_time;
+        for (const RankedVariant &r : ranked)
+            if (!settled && std::memcmp(&r.v, &v, sizeof v) == 0) t.time_major = r.time_major;
         const dd_status s = time_tables(t, ms);
         free_fwd_tables(&t);
         return s;
     };
     auto pick_order = [&](const dd_variant &v) -> dd_status {
         double ms_dm = -1.0, ms_tm = -1.0;
+        settled = true;
         order_time = false;
         dd_status s = time_ms(v, &ms_dm);
         if (s == DD_OK) {
@@ -220,7 +225,7 @@ extern "C" dd_status dd_tune(dd_plan p, int32_t budget_ms, dd_tune_report *rep) 
     const double flop = double(p->B) * p->D * double(p->S) * p->C;
     dd_variant best{};
     std::vector<dd_variant> extra;
-    for (const RankedVariant &r : ranked_variants(p)) extra.push_back(r.v);
+    for (const RankedVariant &r : ranked) extra.push_back(r.v);
     dd_status s = sweep_variants(budget_ms, flop, time_ms, &best, rep, pick_order, extra);
     FwdTables t;
     if (s == DD_OK) s = build_fwd_tables(p, best, &t);
@@ -238,14 +243,27 @@ extern "C" dd_status dd_tune(dd_plan p, int32_t budget_ms, dd_tune_report *rep) 
         s = time_tables(t, &ms_time);
         t.time_major = s == DD_OK && ms_time < ms_dm;
     }
+    // The plan's variant in its order stays if the sweep found nothing faster (a
+    // budget that ended the sweep early, or a variant outside the grid).
+    double ms_now = 0.0;
+    if (s == DD_OK) s = time_tables(p->fwd, &ms_now);
     cleanup();
     if (s != DD_OK) {
         free_fwd_tables(&t);
         return s;
     }
-    if (rep && t.time_major) {
-        rep->best_ms = ms_time;
-        rep->best_gflops = flop / (ms_time * 1e6);
+    const double ms_best = t.time_major ? ms_time : ms_dm;
+    const bool stay = ms_now < ms_best;
+    if (rep && (stay || t.time_major)) {
+        rep->best = stay ? p->fwd.v : best;
+        rep->best_ms = stay ? ms_now : ms_time;
+        rep->best_gflops = flop / (rep->best_ms * 1e6);
+    }
+    if (stay) {
+        free_fwd_tables(&t);
+        p->chosen = true;
+        cache_store(plan_signature(p), p->fwd.v, p->fwd.time_major);
+        return DD_OK;
     }
     s = replace_fwd_tables(p, &p->fwd, t);
     if (s != DD_OK) return s;

@@ -15,7 +15,7 @@ typedef struct {
     unsigned char arg0[256];
 } launch_t;
 
-static launch_t launches[64];
+static launch_t launches[64], last;
 static int n_launches;
 
 int fake_launch_count(void) { return n_launches; }
@@ -77,7 +77,25 @@ err_t cudaGraphExecDestroy(void *e) { return 0; }
 err_t cudaGraphDestroy(void *g) { return 0; }
 err_t cudaGetLastError(void) { return 0; }
 err_t __cudaGetKernel(void **k, const void *f) { *k = (void *)f; return 0; }
+/* Milliseconds of the last forward launch, by its tile and launch order: 0.5 for
+ * the favoured tile with time tiles fastest, 2 for it with DM tiles fastest, 1.5
+ * and 1 for the others. (Offsets of FwdArgs: see fake_gpu.py.) */
+static int favoured[3];
+void fake_favour(int dt, int ts, int cch) {
+    favoured[0] = dt;
+    favoured[1] = ts;
+    favoured[2] = cch;
+}
+err_t cudaEventElapsedTime(float *ms, void *a, void *b) {
+    int shape[4], order;
+    memcpy(shape, last.arg0 + 48, sizeof shape); /* Dt, Ts, C_pad, cch */
+    memcpy(&order, last.arg0 + 108, sizeof order);
+    const int hit = shape[0] == favoured[0] && shape[1] == favoured[1] && shape[3] == favoured[2];
+    *ms = hit ? (order ? 0.5f : 2.0f) : (order ? 1.5f : 1.0f);
+    return 0;
+}
 err_t __cudaLaunchKernel(void *f, dim3_t grid, dim3_t block, void **args, size_t smem, void *s) {
+    if (smem) memcpy(last.arg0, args[0], sizeof last.arg0);
     if (n_launches < 64) {
         launch_t *l = &launches[n_launches++];
         l->grid = grid;

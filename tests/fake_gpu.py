@@ -109,6 +109,17 @@ def _child():
         with open(os.environ["DD_TUNE_CACHE"], "a") as f:
             f.write(" ".join([key] + [str(x) for x in entry]) + "\n")
 
+    def tuned(p):
+        """What dd_tune settles on where the plan's own tile and order are the
+        fastest there is, and the tile in the other order the slowest."""
+        v = L.Variant()
+        L.check(lib.dd_plan_get_variant(p, ctypes.byref(v)))
+        fake.fake_favour(v.dm_per_thread * v.warps_dm, 32 * v.samples_per_thread * v.warps_time,
+                         v.chans_per_stage)
+        rep = L.TuneReport()
+        L.check(lib.dd_tune(p, 400, ctypes.byref(rep)))
+        return [variant(lib.dd_plan_get_variant, p), order(p), list(rep.best.as_tuple()), rep.best_ms]
+
     answers = []
     buf = ctypes.create_string_buffer(4096)
     ptr = ctypes.c_void_p((ctypes.addressof(buf) + 255) & ~255)
@@ -131,6 +142,8 @@ def _child():
                                         (ctypes.c_void_p * len(plans))(*[p.value for p in plans])))
             ans["batch"] = variant(lib.dd_batch_get_variant, b)
             lib.dd_batch_destroy(b)
+        if "tune" in ask:
+            ans["tuned"] = tuned(plans[0])
         if "stream" in ask:
             s = ctypes.c_void_p()
             L.check(lib.dd_stream_create(ctypes.byref(s), plans[0]))

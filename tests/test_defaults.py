@@ -125,3 +125,12 @@ def test_stream_fill_covers_the_machine(tmp_path, setup, least):
     fill = probe([{"setups": [setup], "ask": ["stream"]}], tmp_path)[0]["stream_launches"][0]
     assert fill["smem"] == 0 and fill["grid"][0] == setup[1] * setup[2]
     assert least <= fill["grid"][0] * fill["grid"][1] <= max(least, 16 * 152), fill
+
+
+def test_tuner_times_candidates_in_their_own_order(tmp_path):
+    """A default that is fast only with time tiles fastest is not given up for
+    a slower variant."""
+    got = probe([{"setups": [("lofar", 1, 32, 64, 100000, "f32")], "ask": ["tune"]}], tmp_path)[0]
+    assert got["orders"] == [1], got
+    v, order, best, ms = got["tuned"]
+    assert order == 1 and best == v and ms == 0.5 and v[:5] == got["plans"][0][:5], got
