@@ -275,11 +275,6 @@ int worklist_pos(const dd_batch_s *bt, int u) {
     return -1;
 }
 
-double tile_cost(dd_plan p) {
-    const FwdTables &t = p->fwd;
-    return double(p->C) * t.Dt * t.Ts;
-}
-
 }  // namespace
 }  // namespace dd
 
@@ -301,8 +296,10 @@ dd_status dd_batch_create(dd_batch *out, int32_t n, const dd_plan *plans) {
     if (!bt) return fail(DD_ERR_NOMEM, "host allocation");
     std::vector<int> idx(static_cast<size_t>(n), 0);
     for (int i = 0; i < n; ++i) idx[size_t(i)] = i;
+    // Heaviest tile first: the batch starts with one tile shape for all plans, so
+    // the one with the most channels (the plans' own tiles say nothing here).
     std::stable_sort(idx.begin(), idx.end(),
-                     [&](int x, int y) { return tile_cost(plans[x]) > tile_cost(plans[y]); });
+                     [&](int x, int y) { return plans[x]->C > plans[y]->C; });
     for (int i : idx) {
         bt->plans.push_back(plans[i]);
         bt->user_index.push_back(i);

@@ -60,6 +60,7 @@ def _child():
     lib = L.load()
     fake = ctypes.CDLL(os.environ["FAKE_CUDART"])
     fake.fake_launch.restype = ctypes.POINTER(Launch)
+    fake.fake_upload.restype = ctypes.c_void_p
 
     def plan(band, beams, chan, dm, out, dtype):
         lo, hi, t_samp, step = BANDS[band]
@@ -109,6 +110,15 @@ def _child():
         with open(os.environ["DD_TUNE_CACHE"], "a") as f:
             f.write(" ".join([key] + [str(x) for x in entry]) + "\n")
 
+    def work_list(b, n):
+        """Channels of the plans in the order that a batch's launch takes them."""
+        bufs = (ctypes.c_void_p * n)(*[ptr.value] * n)
+        L.check(lib.dd_batch_execute(b, bufs, bufs, bufs, None))
+        size = ctypes.c_size_t()
+        raw = ctypes.string_at(fake.fake_upload(ctypes.byref(size)), size.value)
+        step = size.value // n
+        return [FwdArgsHead.from_buffer_copy(raw[i * step:]).C for i in range(n)]
+
     def tuned(p):
         """What dd_tune settles on where the plan's own tile and order are the
         fastest there is, and the tile in the other order the slowest."""
@@ -141,6 +151,7 @@ def _child():
             L.check(lib.dd_batch_create(ctypes.byref(b), len(plans),
                                         (ctypes.c_void_p * len(plans))(*[p.value for p in plans])))
             ans["batch"] = variant(lib.dd_batch_get_variant, b)
+            ans["batch_channels"] = work_list(b, len(plans))
             lib.dd_batch_destroy(b)
         if "tune" in ask:
             ans["tuned"] = tuned(plans[0])

@@ -134,3 +134,13 @@ def test_tuner_times_candidates_in_their_own_order(tmp_path):
     assert got["orders"] == [1], got
     v, order, best, ms = got["tuned"]
     assert order == 1 and best == v and ms == 0.5 and v[:5] == got["plans"][0][:5], got
+
+
+def test_batches_take_the_longest_tiles_first(tmp_path):
+    """All plans of a batch run tiles of one shape: those with the most channels
+    come first, whatever tiles the plans take on their own."""
+    setups = [["lband", 96, 64, 64, 4096, "u8"], ["lband", 1, 100, 20, 1000, "u8"],
+              ["lowfreq", 4, 208, 500, 4000, "u8"]]
+    got = probe([{"setups": setups, "ask": ["batch"]}, {"setups": setups[:2], "ask": ["batch"]}],
+                tmp_path)
+    assert [g["batch_channels"] for g in got] == [[208, 100, 64], [100, 64]]
