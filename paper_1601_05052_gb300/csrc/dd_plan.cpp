@@ -62,7 +62,8 @@ dd_status check_variant_shape(const dd_variant &v) {
     const bool wide = is_wide(v.kind, v.dm_per_thread, v.samples_per_thread);
     const int cch = v.chans_per_stage;
     if (cch != 4 && cch != 8 && cch != 16 && cch != 32 && !(wide && (cch == 1 || cch == 2)))
-        return fail(DD_ERR_ARG, "variant chans_per_stage must be 4, 8, 16 or 32");
+        return fail(DD_ERR_ARG, "variant chans_per_stage must be 4, 8, 16 or 32 (wide kernels: 1 "
+                                "and 2 too)");
     if (v.stages < 2 || v.stages > 4) return fail(DD_ERR_ARG, "variant stages must be 2..4");
     return DD_OK;
 }

@@ -19,7 +19,8 @@ BANDS = {"lband": (1400.0, 1500.0, 64e-6, 0.5), "apertif": (1420.0, 1720.0, 50e-
 
 def probe(requests, tmp_path):
     """Answers of the child to each request {"setups": [[band, beams, channels,
-    trials, samples, type], ...], "set": variant of the first plan, "transposed": variant and launch order that
+    trials, samples, type], ...], "set": variant of the first plan,
+    "refuse": variant that it refuses, "transposed": variant and launch order that
     a tuning cache holds for its adjoint's plan, "ask": [...]}."""
     from paper_1601_05052_gb300 import _build
     _build.build()
@@ -140,6 +141,9 @@ def _child():
         ask = req.get("ask", [])
         if "set" in req:
             L.check(lib.dd_plan_set_variant(plans[0], ctypes.byref(L.Variant(*req["set"]))))
+        if "refuse" in req:
+            assert lib.dd_plan_set_variant(plans[0], ctypes.byref(L.Variant(*req["refuse"])))
+            ans["message"] = lib.dd_last_error_message().decode()
         if "transposed" in req:
             cache_transposed(plans[0], req["setups"][0], req["transposed"])
         if "adjoint" in ask:

@@ -144,3 +144,11 @@ def test_batches_take_the_longest_tiles_first(tmp_path):
     got = probe([{"setups": setups, "ask": ["batch"]}, {"setups": setups[:2], "ask": ["batch"]}],
                 tmp_path)
     assert [g["batch_channels"] for g in got] == [[208, 100, 64], [100, 64]]
+
+
+def test_refusals_name_what_is_accepted(tmp_path):
+    """Chunks of 1 and 2 channels exist for the wide kernels only; the refusal
+    of another size says so."""
+    bad = [[0, 8, 8, 1, 8, 3, 3], [0, 4, 8, 4, 1, 2, 3]]
+    for a in probe([{"setups": [list(LBAND96) + ["f32"]], "refuse": v} for v in bad], tmp_path):
+        assert "4, 8, 16 or 32" in a["message"] and "1 and 2" in a["message"], a
