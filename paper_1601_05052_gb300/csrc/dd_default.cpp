@@ -11,18 +11,18 @@
 // once; staged bytes (L2) and compulsory bytes (HBM) bound the sum from below.
 // (Lane-strided with two small slots: latency s more, as no copy is in flight
 // while a chunk is summed.)
-// The constants of each kernel family were fitted on a GB300 to 66900 timings
-// (44 variants, where they fit, on 2439 setups: 2036 drawn from five bands, 1 to
-// 384 beams, 16 to 1024 channels, 4 to 2048 trials, all input types, the
-// gradients' transposed tables too; 403 at steps of up to 1.5 samples), then
-// adjusted, on four fifths of the setups, to what the choice costs. Residuals
-// 11 % (windows) to 20 % (kind 4). The choice, among the variants that keep a
-// plan's channel groups (dd_plan.cpp), takes 1.017 times the best one's time in
-// the geometric mean (1.017 on the last fifth too), 1.12 at the 95th percentile
-// and 1.63 at worst. (1.041 and 2.67 with register counts that ptxas
-// contradicts, corrected by rules on channels, trials and steps.)
+// The constants of each kernel family were fitted on a GB300 to 75700 timings
+// (44 variants, where they fit, on 3550 setups: 2036 drawn from five bands, 1 to
+// 384 beams, 16 to 1024 channels, 4 to 2048 trials, all input types, some
+// gradients' transposed tables; 403 at steps of up to 1.5 samples; 1111
+// transposed tables at 120-180 and 138-144 MHz), then adjusted, on four fifths
+// of the setups, to what the choice costs. Residuals 9 % (quads) to 21 % (kind
+// 2). The choice, among the variants that keep a plan's channel groups
+// (dd_plan.cpp), takes 1.018 times the best one's time in the geometric mean
+// (1.018 on the last fifth too), 1.11 at the 95th percentile and 1.63 at worst.
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 
 #include "dd_internal.h"
 
@@ -35,7 +35,7 @@ struct Candidate {
     bool time_major;
 };
 
-// The variants worth starting with: the best of them takes 1.005 times the best
+// The variants worth starting with: the best of them takes 1.003 times the best
 // of all 44 in the geometric mean.
 const Candidate kCandidates[] = {
     // sub-bands: long Eq. 1 grids whose channel groups share delay patterns
@@ -83,13 +83,13 @@ const Candidate kCandidates[] = {
 struct Fit {
     double a, b, k, l, o, s, m;
 };
-constexpr Fit kLane{1.02, 0.47, 1.3, 3.01, 7.05, 128.67, 13.03};
-constexpr Fit kQuad{0.92, 20.68, 3.34, 23.41, 11.85, 0, 10.12};
-constexpr Fit kWindow{1.08, 1.32, 10.44, 39.46, 8.79, 0, 10.97};
-constexpr Fit kReuse{0.6, 5.15, 20, 13.09, 8.18, 0, 35.74};
-constexpr Fit kSub2{1.81, 0.17, 12.18, 17.93, 6.43, 2.09, 19.16};
-constexpr Fit kSub4{0.82, 5.23, 3.48, 18.56, 8.44, 6.35, 6.62};
-constexpr Fit kSub6{1.28, 0.83, 0.72, 5.08, 9.39, 7.49, 0.51};
+constexpr Fit kLane{1.02, 1.2, 1.31, 2.56, 6.08, 129.99, 14.66};
+constexpr Fit kQuad{1.09, 19.26, 3.89, 25.72, 9.8, 0, 12.39};
+constexpr Fit kWindow{1.08, 4.28, 8.06, 25.66, 8.62, 0, 23.07};
+constexpr Fit kReuse{0.63, 14.59, 1.64, 24.87, 8.86, 0, 15.3};
+constexpr Fit kSub2{0.96, 0.35, 11.67, 19.14, 8.39, 6.37, 20.33};
+constexpr Fit kSub4{0.69, 6.59, 2.42, 20.76, 7.41, 6.88, 3.37};
+constexpr Fit kSub6{1.33, 0.7, 0.47, 18.82, 7.66, 8.78, 5.21};
 
 // Registers per thread of the candidates' one-shot kernels, as ptxas reports
 // them (asking the runtime would load every candidate's code at plan time).
@@ -109,12 +109,16 @@ int registers(dd_dtype t, const dd_variant &v) {
 
 DelaySteps delay_steps(const dd_plan_s *p) {
     DelaySteps s;
+    const int K = std::min(p->D - 1, 16);  // trials of a small tile
     std::vector<int32_t> lo(p->shifts.begin(), p->shifts.begin() + p->C), hi = lo;
+    int32_t span = 0;
     for (int d = 1; d < p->D; ++d) {
         const int32_t *row = &p->shifts[size_t(d) * p->C];
+        const int32_t *back = d >= K ? row - size_t(K) * p->C : row;
         for (int c = 0; c < p->C; ++c) {
             lo[size_t(c)] = std::min(lo[size_t(c)], row[c]);
             hi[size_t(c)] = std::max(hi[size_t(c)], row[c]);
+            span = std::max(span, std::abs(row[c] - back[c]));
         }
     }
     for (int c = 0; c < p->C; ++c) {
@@ -122,6 +126,7 @@ DelaySteps delay_steps(const dd_plan_s *p) {
         s.mean += x / p->C;
         s.max = std::max(s.max, x);
     }
+    s.widest = double(span) / std::max(1, K);
     return s;
 }
 
@@ -142,12 +147,12 @@ double model_us(const dd_plan_s *p, const DelaySteps &st, const dd_variant &v) {
     const double tiles = std::ceil(double(p->D) / Dt) * std::ceil(double(p->S) / Ts) * p->B;
     // window of a channel for the tile's trials, in a mean and the widest channel
     const double len = std::min(Ts + (De - 1) * st.mean, De * Ts);
-    const double widest = std::min(Ts + (De - 1) * st.max, De * Ts);
+    const double widest = std::min(Ts + (De - 1) * st.widest, De * Ts);
     // resident CTAs per SM
     const double slot = std::min(cch, C) * widest * elt + cch * (2 * Dt + 20);
     double smem = 1152 + v.stages * slot;
     if (sb) {  // partial series, at five patterns per group
-        const double series = cch / 4 * 5 * (Ts + De * st.max) * 4 * 1.15;
+        const double series = cch / 4 * 5 * (Ts + De * st.widest) * 4 * 1.15;
         smem += v.kind == 6 ? series : 2 * series;
     }
     const int threads = 32 * (nw + extra_warps(v.kind));

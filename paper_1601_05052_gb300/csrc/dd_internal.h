@@ -213,9 +213,11 @@ dd_status launch_adjoint(dd_plan_s *p, const float *g, const float *w, const flo
                          float *gin, float *gw, cudaStream_t st);
 
 // Default variants (dd_default.cpp). Delay steps: how far a channel's delay
-// moves per trial, mean and largest over the channels.
+// moves per trial over all trials, mean and largest over the channels; and the
+// largest over any 16 trials, which sizes the windows (a gradient's transposed
+// table steps unevenly: 1.7 times the mean's largest at 120-180 MHz).
 struct DelaySteps {
-    double mean = 0, max = 0;
+    double mean = 0, max = 0, widest = 0;
 };
 DelaySteps delay_steps(const dd_plan_s *p);
 double model_us(const dd_plan_s *p, const DelaySteps &st, const dd_variant &v);

@@ -152,3 +152,14 @@ def test_refusals_name_what_is_accepted(tmp_path):
     bad = [[0, 8, 8, 1, 8, 3, 3], [0, 4, 8, 4, 1, 2, 3]]
     for a in probe([{"setups": [list(LBAND96) + ["f32"]], "refuse": v} for v in bad], tmp_path):
         assert "4, 8, 16 or 32" in a["message"] and "1 and 2" in a["message"], a
+
+
+@pytest.mark.parametrize("setup", [("lowfreq", 5, 95, 220, 2494, "f32"),
+                                   ("lowfreq", 6, 74, 121, 2801, "f32"),
+                                   ("lowfreq", 3, 111, 266, 5410, "f32")], ids=str)
+def test_adjoint_windows_are_sized_by_the_widest_steps(tmp_path, setup):
+    """A transposed table steps unevenly: tiles of 8 trials x 512 samples, which
+    the mean step lets two blocks per SM hold, are 1.7 times slower there than
+    4 x 1024 (165 us against 276 for the first)."""
+    got = probe([{"setups": [setup], "ask": ["adjoint"]}], tmp_path)[0]
+    assert got["adjoint"][:5] == [0, 4, 8, 1, 4] or got["adjoint"][:5] == [0, 4, 8, 1, 8], got
