@@ -258,10 +258,7 @@ dd_status configure_default(dd_batch_s *bt) {
             const bool chain = !sums_groups(v.kind, v.dm_per_thread, v.samples_per_thread);
             if (chain && !looked) {
                 looked = true;
-                for (size_t j = 0; j < bt->plans.size() && !keep; ++j) {
-                    const dd_status q = keeps_groups(bt->plans[j], &keep);
-                    if (q != DD_OK) return q;
-                }
+                keep = std::any_of(bt->plans.begin(), bt->plans.end(), keeps_groups);
             }
             if (chains == 0 ? !(chain && keep) : chain && keep) s = configure(bt, v);
         }

@@ -230,7 +230,7 @@ struct RankedVariant {
 // The candidate variants, fastest by the model first (they may not fit).
 std::vector<RankedVariant> ranked_variants(const dd_plan_s *p);
 // Whether defaults of this plan must sum groups of four channels (dd_plan.cpp).
-dd_status keeps_groups(dd_plan_s *p, bool *keeps);
+bool keeps_groups(dd_plan_s *p);
 
 bool aligned16(const void *p);
 

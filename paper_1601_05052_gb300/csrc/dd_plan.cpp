@@ -534,19 +534,84 @@ void cache_store(const std::string &key, const dd_variant &v, bool time_major) {
 
 namespace {
 
-// Builds the preference list's first sub-band variant that fits a float plan;
-// DD_ERR_ARG if none does (or for 8-bit input, whose sums are exact in any
-// order). Remembers which in p->groups.
-dd_status build_list_subband(dd_plan_s *p, FwdTables *out) {
-    dd_status s = DD_ERR_ARG;
-    for (const dd_variant &d : kDefaults) {
-        if (p->dtype == DD_U8 || !is_subband(d.kind)) break;
-        s = build_fwd_tables(p, d, out);
-        if (s != DD_ERR_ARG) break;
-    }
-    if (s == DD_OK || s == DD_ERR_ARG) p->groups = s == DD_OK;
-    return s;
+// Whether a sub-band variant fits a float plan: its tables' conditions without
+// the tables, which take ten times as long. *patterns: whether the delay patterns
+// per group and tile are few enough.
+bool subband_fits(const dd_plan_s *p, const dd_variant &v, bool *patterns) {
+    const int Dt = v.dm_per_thread * v.warps_dm, cch = v.chans_per_stage;
+    const int Ts = 32 * v.samples_per_thread * v.warps_time;
+    const int64_t al = align_elems(p->dtype), elt = elt_bytes(p->dtype);
+    int64_t stage_max = 0, p_max = 0, blocks_max = 0;
+    *patterns = false;
+    for (int d0 = 0; d0 < p->D; d0 += Dt)
+        for (int c0 = 0; c0 < p->C; c0 += cch) {
+            int64_t stage = 0, series = 0, blocks = 0;
+            for (int ga = c0; ga < std::min(p->C, c0 + cch); ga += kSbGroup) {
+                const int gn = std::min(kSbGroup, p->C - ga), ref = gn - 1;
+                int32_t pat[kSbPatterns][kSbGroup], bmin[kSbPatterns], bmax[kSbPatterns];
+                int32_t lo[kSbGroup], hi[kSbGroup];
+                int n = 0;
+                for (int d = d0; d < std::min(p->D, d0 + Dt); ++d) {
+                    const int32_t *sh = &p->shifts[size_t(d) * p->C + ga];
+                    int q = 0;
+                    for (; q < n; ++q) {
+                        bool same = true;
+                        for (int j = 0; j < ref; ++j) same &= sh[j] - sh[ref] == pat[q][j];
+                        if (same) break;
+                    }
+                    if (q == kSbPatterns) return false;
+                    if (q == n) {
+                        for (int j = 0; j < ref; ++j) pat[q][j] = sh[j] - sh[ref];
+                        bmin[n] = bmax[n] = sh[ref];
+                        ++n;
+                    }
+                    bmin[q] = std::min(bmin[q], sh[ref]);
+                    bmax[q] = std::max(bmax[q], sh[ref]);
+                    for (int j = 0; j < gn; ++j) {
+                        lo[j] = d == d0 ? sh[j] : std::min(lo[j], sh[j]);
+                        hi[j] = d == d0 ? sh[j] : std::max(hi[j], sh[j]);
+                    }
+                }
+                for (int q = 0; q < n; ++q) {
+                    const int64_t len = int64_t(bmax[q]) - bmin[q] + Ts;
+                    series += round_up(len, 32);
+                    blocks += (len + 127) / 128;
+                }
+                for (int j = 0; j < gn; ++j) {
+                    const int64_t ws = floor_to(lo[j], al);
+                    stage += round_up(hi[j] + Ts - ws, al);
+                }
+            }
+            stage_max = std::max(stage_max, stage);
+            p_max = std::max(p_max, series);
+            blocks_max = std::max(blocks_max, blocks);
+        }
+    *patterns = true;
+    const int64_t offs = cch / kSbGroup * Dt * 2;
+    const int64_t slot = round_up((stage_max + 64) * elt, 16) + offs + blocks_max * 16 + cch * 4;
+    const int64_t smem =
+        128 + v.stages * slot + (v.kind == 6 ? 1 : 2) * (round_up(p_max + 64, 4) * 4 + offs);
+    return stage_max <= 65536 && p_max <= 65536 - Ts && smem <= int64_t(p->smem_optin);
 }
+
+// Whether one of the preference list's sub-band variants fits, the one with the
+// fewest trials per tile first: patterns that are too many for it are too many
+// for all.
+bool list_subband_fits(const dd_plan_s *p) {
+    bool patterns = true;
+    for (int i = int(sizeof(kDefaults) / sizeof(kDefaults[0])) - 1; i >= 0 && patterns; --i)
+        if (is_subband(kDefaults[i].kind) && subband_fits(p, kDefaults[i], &patterns)) return true;
+    return false;
+}
+
+}  // namespace
+
+bool keeps_groups(dd_plan_s *p) {
+    if (p->groups < 0) p->groups = p->dtype != DD_U8 && list_subband_fits(p);
+    return p->groups == 1;
+}
+
+namespace {
 
 // The tables a plan starts with: the modelled candidates in their order, then
 // the preference list; DD_ERR_ARG if none fits. A float plan that a sub-band
@@ -555,31 +620,16 @@ dd_status build_list_subband(dd_plan_s *p, FwdTables *out) {
 // for the plans that have no such variant (384 beams x 64 channels x 4 trials:
 // largest error 8.2e-8 of the largest output in groups, 1.7e-7 in one chain).
 dd_status build_default(dd_plan_s *p, FwdTables *out) {
-    FwdTables sub;  // the list's sub-band variant, once a chain stands next
     dd_status s = DD_ERR_ARG;
     for (const RankedVariant &r : ranked_variants(p)) {
-        const dd_variant &v = r.v;
-        const bool chain = !sums_groups(v.kind, v.dm_per_thread, v.samples_per_thread);
-        if (chain && p->groups < 0) {
-            s = build_list_subband(p, &sub);
-            if (s != DD_OK && s != DD_ERR_ARG) return s;
-        }
-        if (chain && p->groups == 1) continue;
-        if (p->groups == 1 && std::memcmp(&v, &sub.v, sizeof v) == 0) {
-            *out = sub;
-            return DD_OK;
-        }
-        s = build_fwd_tables(p, v, out);
+        if (!sums_groups(r.v.kind, r.v.dm_per_thread, r.v.samples_per_thread) && keeps_groups(p))
+            continue;
+        s = build_fwd_tables(p, r.v, out);
         if (s == DD_ERR_ARG) continue;
-        if (p->groups == 1) free_fwd_tables(&sub);
         out->time_major = s == DD_OK && r.time_major;
         return s;
     }
-    if (p->groups == 1) {
-        *out = sub;
-        return DD_OK;
-    }
-    for (const dd_variant &d : kDefaults) {
+    for (const dd_variant &d : kDefaults) {  // sub-bands first
         s = build_fwd_tables(p, d, out);
         if (s != DD_ERR_ARG) return s;
     }
@@ -643,18 +693,6 @@ dd_status check_common(dd_plan *out, int32_t n_chan, int32_t n_dm, int64_t n_out
 }
 
 }  // namespace
-
-dd_status keeps_groups(dd_plan_s *p, bool *keeps) {
-    if (p->groups < 0) {
-        FwdTables t;
-        const dd_status s = build_list_subband(p, &t);
-        if (s == DD_OK) free_fwd_tables(&t);
-        if (s != DD_OK && s != DD_ERR_ARG) return s;
-    }
-    *keeps = p->groups == 1;
-    return DD_OK;
-}
-
 }  // namespace dd
 
 using namespace dd;

@@ -19,7 +19,7 @@ BANDS = {"lband": (1400.0, 1500.0, 64e-6, 0.5), "apertif": (1420.0, 1720.0, 50e-
 
 def probe(requests, tmp_path):
     """Answers of the child to each request {"setups": [[band, beams, channels,
-    trials, samples, type], ...], "set": variant of the first plan,
+    trials, samples, type], ...] or "tables": [[delays, samples, type], ...], "set": variant of the first plan,
     "refuse": variant that it refuses, "transposed": variant and launch order that
     a tuning cache holds for its adjoint's plan, "ask": [...]}."""
     from paper_1601_05052_gb300 import _build
@@ -120,6 +120,23 @@ def _child():
         step = size.value // n
         return [FwdArgsHead.from_buffer_copy(raw[i * step:]).C for i in range(n)]
 
+    def fits_and_keeps(table, out, dtype):
+        """Whether a sub-band variant of the preference list fits a delay
+        table's plan, and whether the library says that its sums keep groups."""
+        chan, dm = len(table[0]), len(table)
+        sh = (ctypes.c_int32 * (chan * dm))(*[x for row in table for x in row])
+        p = ctypes.c_void_p()
+        L.check(lib.dd_plan_create_from_shifts(ctypes.byref(p), chan, dm, sh, out, 1,
+                                               L.DTYPES[dtype]))
+        keeps = getattr(lib, "_ZN2dd12keeps_groupsEP9dd_plan_s")
+        keeps.restype = ctypes.c_bool
+        fits = [lib.dd_plan_set_variant(p, ctypes.byref(L.Variant(*v))) == 0
+                for v in ((6, 4, 8, 16, 1, 32, 2), (4, 4, 8, 16, 1, 16, 2), (2, 8, 4, 8, 1, 16, 2),
+                          (2, 8, 4, 4, 2, 8, 2))]
+        answer = [any(fits), keeps(p)]
+        lib.dd_plan_destroy(p)
+        return answer
+
     def tuned(p):
         """What dd_tune settles on where the plan's own tile and order are the
         fastest there is, and the tile in the other order the slowest."""
@@ -135,6 +152,9 @@ def _child():
     buf = ctypes.create_string_buffer(4096)
     ptr = ctypes.c_void_p((ctypes.addressof(buf) + 255) & ~255)
     for req in json.loads(sys.stdin.read()):
+        if "tables" in req:
+            answers.append([fits_and_keeps(*t) for t in req["tables"]])
+            continue
         plans = [plan(*s) for s in req["setups"]]
         ans = {"plans": [variant(lib.dd_plan_get_variant, p) for p in plans],
                "orders": [order(p) for p in plans]}

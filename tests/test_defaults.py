@@ -1,6 +1,7 @@
 """What plans start with, decided without a GPU (fake_gpu.py): float sums keep
 the grouping that the sub-band kernels give them, and the time model orders
 setups whose fastest variants are known from timings."""
+import numpy as np
 import pytest
 
 from fake_gpu import probe
@@ -163,3 +164,31 @@ def test_adjoint_windows_are_sized_by_the_widest_steps(tmp_path, setup):
     4 x 1024 (165 us against 276 for the first)."""
     got = probe([{"setups": [setup], "ask": ["adjoint"]}], tmp_path)[0]
     assert got["adjoint"][:5] == [0, 4, 8, 1, 4] or got["adjoint"][:5] == [0, 4, 8, 1, 8], got
+
+
+def test_group_rule_equals_the_built_tables(tmp_path):
+    """The quick look at a delay table says what building the list's sub-band
+    variants says: Eq. 1 tables, equal patterns with wide spans (shared memory
+    decides), steps in stairs, no order, a single step for all channels."""
+    rng = np.random.default_rng(3)
+    tables = []
+    for i in range(200):
+        C, D, mode = int(rng.integers(1, 70)), int(rng.integers(1, 200)), i % 5
+        if mode == 0:
+            f = rng.uniform(100, 1500) * (1 + np.arange(C) * rng.uniform(0.01, 0.3) / C)
+            d = np.arange(D) * rng.uniform(0.01, 2) * 4.148808e3 / 10 ** rng.uniform(-5.3, -3.5)
+            sh = np.floor(d[:, None] * (f ** -2.0 - f[-1] ** -2.0) + 0.5)
+        elif mode == 1:
+            sh = np.sort(rng.integers(0, rng.integers(1, 2000), (D, C)), axis=0)
+        elif mode == 2:
+            sh = rng.integers(0, rng.integers(1, 4000), (D, 1)) + rng.integers(0, 2, (1, C))
+        elif mode == 3:
+            sh = ((np.arange(D) // rng.integers(1, 8) * rng.integers(1, 300))[:, None]
+                  + rng.integers(0, rng.integers(1, 3000), (1, C)))
+        else:
+            sh = np.arange(D)[:, None] * rng.integers(0, 400) + np.zeros((1, C))
+        tables.append([np.minimum(sh, 1 << 26).astype(int).tolist(), int(rng.integers(1, 3000)),
+                       ["f32", "f16"][i % 2]])
+    got = probe([{"tables": tables}], tmp_path)[0]
+    assert 40 <= sum(f for f, _ in got) <= 160
+    assert [i for i, (f, k) in enumerate(got) if f != k] == []
