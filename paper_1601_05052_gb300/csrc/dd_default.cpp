@@ -184,6 +184,12 @@ double model_us(const dd_plan_s *p, const DelaySteps &st, const dd_variant &v) {
     double us = clk / 2070.0;
     us = std::max(us, tiles * C * len * elt / 7.5e6);
     us = std::max(us, (p->B * C * double(p->stride) * elt + 4.0 * p->B * p->D * double(p->S)) / 5.5e6);
+    // Narrow input: one partial-sum slot comes after two of the same size, for
+    // where those do not fit (survey scale, 8-bit: kind 4 2.26 ms, kind 6 2.38;
+    // 439 channels x 287 trials x 19105 samples, FP16: kind 6 203 us, kind 4 with
+    // 16 channels per chunk 225).
+    if (v.kind == 6 && v.warps_dm == 16 && p->dtype != DD_F32)
+        us = std::max(us, 1.0001 * model_us(p, st, {4, 4, 8, 16, 1, 32, 2}));
     return us;
 }
 
@@ -213,9 +219,6 @@ std::vector<RankedVariant> ranked_variants(const dd_plan_s *p) {
         // Windows want 32-bit samples (narrower ones at odd strides collide in
         // the banks: 64 channels x 64 trials, 8-bit, 22.6 against 9.4 us).
         if (is_window(c.v.kind, c.v.samples_per_thread) && p->dtype != DD_F32) continue;
-        // One partial-sum slot only where two do not fit (survey scale, 8-bit:
-        // kind 4 2.26 ms, kind 6 2.38; FP32 fits 32 channels in kind 6 alone).
-        if (c.v.kind == 6 && c.v.warps_dm == 16 && p->dtype != DD_F32) continue;
         r.push_back(RankedVariant{c.v, c.time_major, model_us(p, st, c.v)});
     }
     // 8-bit sums at nearly constant delays: sub-bands first, whose few series

@@ -60,6 +60,9 @@ KNOWN = [
     (("lband", 96, 64, 64, 4096, "f32"), [[5, 4, 22]], 0),
     (("lband", 96, 64, 64, 4096, "u8"), [[0, 4, 20]], 0),
     (("lofar", 1, 32, 2048, 200000, "f32"), [[0, 8, 8]], 1),
+    # two partial-sum slots of 32 channels do not fit, one does (203 against 225 us)
+    (("apertif", 1, 439, 287, 19105, "f16"), [[6, 4, 8]], 0),
+    (("wide", 2, 509, 777, 10001, "f16"), [[4, 4, 8]], 0),
     # one beam, few trials: small tiles (18 to 27 us) against sub-bands (44)
     (("wide", 1, 281, 128, 2189, "f32"), SMALL, 0),
     (("wide", 1, 150, 67, 2091, "f32"), SMALL, 0),
