@@ -445,10 +445,12 @@ struct LaneStrided {
 // channels' products of an output are summed first and then added to its
 // accumulator, a sub-band kernel's operations in the same order, so that both
 // give the same bits and a plan may take either. The reads stay one shared word
-// per add, which bounds the loop as before; 0.98-1.03 times the single chain's
-// time over 27 setups of 4 to 101 trials (384 beams x 64 channels x 4 trials x
-// 4096 samples, FP32: 72.9 -> 72.0 us, largest error 1.7e-7 -> 8.2e-8 of the
-// largest output; one beam, 64 trials: unchanged).
+// per add, which bounds the loop as before: 0.97 to 1.04 of the single chain's
+// speed per tile shape, in the geometric mean over 27 setups of 4 to 101 trials
+// (384 beams x 64 channels x 4 trials x 4096 samples, FP32: 72.9 -> 72.0 us,
+// largest error 1.7e-7 -> 8.2e-8 of the largest output; one beam, 64 trials: 6.6
+// -> 6.4). Two groups are unrolled in the small tiles (2 x 4, 16-bit, one beam:
+// 5.9 -> 5.7 us).
 template <typename T, int DPT, int SPT>
 struct GroupedLanes {
     static constexpr int U = DPT * SPT > 8 ? 1 : 2;  // groups with their loads in flight at once
@@ -1159,9 +1161,9 @@ __device__ __forceinline__ void fwd_tile_sb(const FwdArgs &a, int dtile, int tti
     // number of slots takes about 150 clocks, which every warp waits for), and
     // a lost wait travels with the barrier instead of being read from shared
     // memory after it. Survey scale: FP32 (kind 6) 2.328 -> 2.280 ms, 8-bit
-    // 2.250 -> 2.232 ms. (16-bit input with two slots is the exception: 0.507
-    // ms with the flag, 0.536 with the barrier's answer, at 2 beams x 509
-    // channels x 777 trials x 10001 samples.)
+    // 2.250 -> 2.232 ms. (16-bit input with two slots keeps the flag: with the
+    // barrier's answer the 4 x 8 kernels of kinds 2 and 4 take 1.05 to 1.12 times
+    // as long on each of 26 setups, the 4 x 4 and 8 x 4 ones the same.)
     uint32_t slot = kbase % S, parity = (kbase / S) & 1u;
     for (int k = 0; k < n_chunks; ++k) {
         // A failed wait in any warp is known to all of them after the barrier;

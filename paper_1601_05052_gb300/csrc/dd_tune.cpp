@@ -6,9 +6,9 @@
 // DM) and keeps the configuration with the highest GFLOP/s. Here the sweep
 // covers the compiled variant grid, skipping variants that do not fit the
 // plan or the device, in two passes so that a time budget is spent where it
-// matters: pass 1 times the modelled default candidates (dd_default.cpp) and
-// every (kernel key, CTA shape) at the default staging (8 channels per stage, 3
-// stages); pass 2 times every staging choice for
+// matters: pass 1 times the modelled default candidates (dd_default.cpp, each in
+// its launch order) and every (kernel key, CTA shape) at the default staging (8
+// channels per stage, 3 stages); pass 2 times every staging choice for
 // the three best of pass 1. The report carries the statistics of Section
 // V-B: mean and standard deviation of GFLOP/s over the variants tried, the
 // optimum's distance from the mean in standard deviations ("signal-to-noise
