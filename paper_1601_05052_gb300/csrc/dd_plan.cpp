@@ -535,7 +535,7 @@ void cache_store(const std::string &key, const dd_variant &v, bool time_major) {
 namespace {
 
 // Whether a sub-band variant fits a float plan: its tables' conditions without
-// the tables, which take ten times as long. *patterns: whether the delay patterns
+// the tables, which take about five times as long. *patterns: whether the delay patterns
 // per group and tile are few enough.
 bool subband_fits(const dd_plan_s *p, const dd_variant &v, bool *patterns) {
     const int Dt = v.dm_per_thread * v.warps_dm, cch = v.chans_per_stage;
